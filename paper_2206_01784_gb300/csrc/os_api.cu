@@ -67,9 +67,8 @@ constexpr int kMaxPlaces = 16;  // 64-bit keys in 5-bit digits: 13 places
 
 // Binning kernel variants: tile geometry (4) x digit-ranking method (3);
 // variant v uses geometry v % 4 and ranking v / 4 (0: one ballot per digit
-// bit; 1: adaptive - ballots where the place is skewed, else the hybrid;
-// 2: hybrid - shared-memory lane masks on two of every three batches, ballots
-// on the third).
+// bit; 1: adaptive - ballots where the place is skewed, else counting atomics;
+// 2: counting atomics only).
 // Geometries 0-2 run one block per tile; geometry 3 is the persistent,
 // warp-specialised kernel (os_binning_ws.cuh), for single arrays only.
 constexpr int kGeometries = 4;
@@ -80,20 +79,14 @@ constexpr int kTileConfigs = 3 * kGeometries;
 // os_set_tile_config / os_set_tile_config_bucket (the autotuner's hooks) and
 // read once per sort when it is planned, with atomic loads and stores (a
 // sort may also name its variant itself: os_sort_*_ex).
-// Defaults: geometry 0 with adaptive ranking (the fastest measured on GB300
-// for 32-bit keys at 2^28 across the key distributions), and for 64-bit keys
-// of the largest bucket the persistent warp-specialised geometry with
-// adaptive ranking (64-bit pairs at 2^27: 0.926 against 0.970 ms per pass;
-// 2^24: 0.125 against 0.132; keys only 0.824 against 0.840; 3 % slower on
-// q = 3 keys).
+// Default everywhere: geometry 0 with adaptive ranking, the fastest measured
+// on GB300 for 32- and 64-bit keys from 2^21 keys up (64-bit pairs at 2^27:
+// 0.714 ms per pass against 0.929 with the persistent geometry).
 constexpr int kDefaultTileConfig = kGeometries + 0;
-constexpr int kDefault64LargeConfig = kGeometries + kPersistentGeometry;
 constexpr int kSizeBuckets = 4;  // n < 2^16, < 2^20, < 2^24, larger
 #define OS_FOUR_DEFAULTS {kDefaultTileConfig, kDefaultTileConfig, kDefaultTileConfig, kDefaultTileConfig}
-#define OS_FOUR_DEFAULTS_64 {kDefaultTileConfig, kDefaultTileConfig, kDefaultTileConfig, kDefault64LargeConfig}
-int g_tile_cfg[2][2][kSizeBuckets] = {{OS_FOUR_DEFAULTS, OS_FOUR_DEFAULTS}, {OS_FOUR_DEFAULTS_64, OS_FOUR_DEFAULTS_64}};
+int g_tile_cfg[2][2][kSizeBuckets] = {{OS_FOUR_DEFAULTS, OS_FOUR_DEFAULTS}, {OS_FOUR_DEFAULTS, OS_FOUR_DEFAULTS}};
 #undef OS_FOUR_DEFAULTS
-#undef OS_FOUR_DEFAULTS_64
 
 int size_bucket(uint64_t n) { return n < (1u << 16) ? 0 : n < (1u << 20) ? 1 : n < (1u << 24) ? 2 : 3; }
 

@@ -240,19 +240,19 @@ struct LocalConfig {
 template <int KBITS, bool PAIRS>
 constexpr size_t local_smem_bytes() {
   using L = LocalConfig<KBITS>;
-  return (size_t)L::T * (KBITS / 8) + (PAIRS ? (size_t)L::T * 4 : 0) + (size_t)L::NW * kRadix * 8 + 64 * 4;
+  return (size_t)L::T * (KBITS / 8) + (PAIRS ? (size_t)L::T * 4 : 0) + (size_t)L::NW * kRadix * 4 + 64 * 4;
 }
 
 template <int KBITS, bool PAIRS>
 __global__ void __launch_bounds__(LocalConfig<KBITS>::NT) batch_local_sort_kernel(BatchArgs b) {
   using L = LocalConfig<KBITS>;
   using K = typename KeyWord<KBITS>::type;
-  constexpr int NT = L::NT, IPT = L::IPT, NW = L::NW;
+  constexpr int NT = L::NT, IPT = L::IPT, NW = L::NW, U = rank_chunk(PAIRS, IPT);
   extern __shared__ __align__(128) unsigned char smem[];
   K* kbuf = reinterpret_cast<K*>(smem);
   uint32_t* vbuf = reinterpret_cast<uint32_t*>(smem + (size_t)L::T * sizeof(K));
   uint32_t* whist = reinterpret_cast<uint32_t*>(smem + (size_t)L::T * sizeof(K) + (PAIRS ? (size_t)L::T * 4 : 0));
-  uint32_t* misc = whist + 2 * NW * kRadix;
+  uint32_t* misc = whist + NW * kRadix;
 
   const uint32_t seg = blockIdx.x;
   if (seg >= b.num_segments || b.totals[2]) return;
@@ -266,17 +266,15 @@ __global__ void __launch_bounds__(LocalConfig<KBITS>::NT) batch_local_sort_kerne
   if (PAIRS)
     for (uint32_t i = tid; i < len; i += NT) vbuf[i] = b.vals_in[s0 + i];
 
-  uint32_t* wcnt = whist + NW * kRadix;
-  uint32_t* wmsk = whist + warp * kRadix;
+  uint32_t* wcnt = whist;  // [NW][256] digit counts
   uint32_t* wc = wcnt + warp * kRadix;
   const uint32_t wbase = (uint32_t)warp * IPT * 32 + lane;
-  const uint32_t lane_bit = 1u << lane;
   for (int pass = 0; pass < b.num_places; ++pass) {
     const int shift = b.begin_bit + 8 * pass;
     const int width = min(8, b.end_bit - shift);
     const uint32_t mask = (1u << width) - 1u;
     const uint32_t dxor = (pass == b.num_places - 1 ? b.top_xor : 0u) ^ (b.descending ? mask : 0u);
-    for (int i = tid; i < 2 * NW * kRadix; i += NT) whist[i] = 0;
+    for (int i = tid; i < NW * kRadix; i += NT) whist[i] = 0;
     __syncthreads();  // staged keys (or the previous pass's scatter) visible
     K key[IPT];
     const K first = kbuf[0];
@@ -292,19 +290,27 @@ __global__ void __launch_bounds__(LocalConfig<KBITS>::NT) batch_local_sort_kerne
 
     uint32_t rank[IPT];
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      const bool valid = wbase + i * 32 < len;
-      rank[i] = wlms_rank<false>(wmsk, wc, digit_of(key[i], shift, mask, dxor), valid, lane_bit, true);
+    for (int i0 = 0; i0 < IPT; i0 += U) {
+      uint32_t d[U], r[U];
+      bool valid[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        valid[u] = wbase + (i0 + u) * 32 < len;
+        d[u] = digit_of(key[i0 + u], shift, mask, dxor);
+      }
+      rank_atomic<false, U>(wc, d, valid, r);
+#pragma unroll
+      for (int u = 0; u < U; ++u) rank[i0 + u] = r[u];
     }
     __syncthreads();
     uint32_t total = 0;
     if (tid < kRadix)
-      for (int w = 0; w < NW; ++w) total += wcnt[w * kRadix + tid];
+      for (int w = 0; w < NW; ++w) total += wcnt[w * kRadix + tid] & 0xFFFFu;  // (the high halves hold lane sums)
     const uint32_t excl = block_exclusive_sum<NT>(tid < kRadix ? total : 0u, misc);
     if (tid < kRadix) {
       uint32_t run = excl;
       for (int w = 0; w < NW; ++w) {
-        const uint32_t cw = wcnt[w * kRadix + tid];
+        const uint32_t cw = wcnt[w * kRadix + tid] & 0xFFFFu;
         wcnt[w * kRadix + tid] = run;
         run += cw;
       }

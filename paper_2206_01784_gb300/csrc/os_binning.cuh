@@ -23,14 +23,13 @@
 //  5. each warp's per-digit counters start at the local position of its
 //     first key of that digit (tile bin start plus the lower warps' counts);
 //  6. warp-level multi-split ranking: each warp walks its keys in 32-wide
-//     batches and finds the lanes holding the same digit, either as in the
-//     paper with one ballot per digit bit ANDed together, or by having every
-//     lane OR its bit into a per-warp shared-memory mask word of its digit
-//     (OR commutes, so the mask read back is exact whatever the order of the
-//     atomics). The lowest lane of each group bumps the warp's counter of the
-//     digit and the group reads the old value (Section 3, WLMS paragraph):
-//     with counters that start at local positions, that is the key's place
-//     in the tile's shared-memory bins, and the key is written there at once.
+//     batches and ranks each among the warp's equal digits, either as in the
+//     paper with one ballot per digit bit ANDed together and the lowest lane
+//     of each group bumping the warp's counter (Section 3, WLMS paragraph), or
+//     with counting atomics whose undefined order among equal lanes is
+//     replaced by lane order (rank_atomic). With counters that start at local
+//     positions, the rank is the key's place in the tile's shared-memory
+//     bins, and the key is written there at once.
 //     Every kRoundEvery batches the look-back's round in flight is folded in
 //     and the next one sent, so its L2 round trips ride along the ranking. A
 //     __match_any_sync per key measured 1.7x slower than the ballots on
@@ -58,29 +57,40 @@ namespace onesweep {
 
 // Tile geometries (threads per block, keys per thread, resident blocks per
 // SM). Index = the geometry part of the launcher's tile configuration.
+// Geometry 0, the default, has the largest tile of which three blocks still
+// fit an SM by registers (80 a thread) and shared memory (76 KB for 32-bit
+// pairs, 72 KB for 64-bit pairs): the look-back's reads, its wait and the
+// per-tile scans are paid per tile, and longer runs write fewer partial lines,
+// while fewer than 24 warps leave the shared-memory pipe idle. Measured at
+// 2^28 u32, ms per pass, pairs / keys only: 256 x 24 x 3 blocks 1.13 / 0.836,
+// 256 x 32 x 3 1.01 / 0.723, 256 x 36 x 3 - / 0.721, 384 x 32 x 2 1.03 /
+// 0.730, 512 x 24 x 2 1.34 / 0.742, 256 x 40 x 2 1.07 / 0.799, 512 x 32 x 1
+// 1.20 / 0.868; at 2^27 u64: 256 x 12 x 3 0.905 / 0.741, 256 x 16 x 3 0.788 /
+// 0.630, 256 x 20 x 3 0.714 / 0.566, 256 x 24 x 2 0.765 / 0.606. The smaller
+// tiles were not faster at any size from 2^21 to 2^25 either.
 template <int KBITS, int CFG> struct TileShape;
-template <> struct TileShape<32, 0> { static constexpr int NT = 256, IPT = 24, MINB = 3; };
+template <> struct TileShape<32, 0> { static constexpr int NT = 256, IPT = 32, MINB = 3; };
 template <> struct TileShape<32, 1> { static constexpr int NT = 256, IPT = 20, MINB = 3; };
 template <> struct TileShape<32, 2> { static constexpr int NT = 256, IPT = 16, MINB = 4; };
-template <> struct TileShape<64, 0> { static constexpr int NT = 256, IPT = 12, MINB = 3; };
+template <> struct TileShape<64, 0> { static constexpr int NT = 256, IPT = 20, MINB = 3; };
 template <> struct TileShape<64, 1> { static constexpr int NT = 256, IPT = 10, MINB = 3; };
 template <> struct TileShape<64, 2> { static constexpr int NT = 256, IPT = 8, MINB = 4; };
 
-// Digit-ranking variants of step 4. Two methods find the lanes sharing a
-// digit: ballots (one per digit bit, the paper's WLMS; ALU work, insensitive
-// to the key distribution) and shared-memory lane masks (every lane ORs its
-// bit into its digit's mask word; shared-memory work that slows down when
-// many lanes share a digit).
+// Digit-ranking variants of step 6. Two methods find a key's rank among the
+// equal digits of its warp: ballots (one per digit bit, the paper's WLMS; ALU
+// work, insensitive to the key distribution) and counting atomics (every lane
+// adds one to its digit's counter and reads it back; shared-memory work that
+// slows down when many lanes share a digit).
 constexpr int kRankBallot = 0;    // ballots only
-constexpr int kRankAdaptive = 1;  // hybrid, or ballots only where the pass's place is skewed
-constexpr int kRankHybrid = 2;    // both methods, by batch (spreads the work over the ALU
-                                  // and shared-memory pipes)
+constexpr int kRankAdaptive = 1;  // counting atomics, or ballots where the pass's place is skewed
+constexpr int kRankAtomic = 2;    // counting atomics only
 
-// Batches of the hybrid ranking that use lane masks: two of every three (the
-// third uses ballots). Measured on GB300 against every other batch, every
-// batch, one in three and one in four: this split is the fastest for 32-bit
-// pairs, keys only and 64-bit pairs.
-__host__ __device__ constexpr bool hybrid_uses_masks(int batch) { return batch % 3 != 0; }
+// Batches whose counting atomics are in flight together: they do not depend
+// on one another, so a chunk pays one shared-memory round trip. Pairs keep
+// their positions in registers beside the keys and take two (2^28 u32 pairs:
+// 1.003 ms per pass against 1.017 with four; keys only 0.727 with two, 0.723
+// with four, 0.716 with eight).
+__host__ __device__ constexpr int rank_chunk(bool pairs, int ipt) { return pairs || ipt % 4 != 0 ? 2 : 4; }
 
 template <int KBITS, bool PAIRS, int CFG = 0>
 struct BinningConfig {
@@ -93,7 +103,7 @@ struct BinningConfig {
   // staging buffers hold a tile plus the slack of a 16-byte-aligned span
   static constexpr size_t kbuf_bytes = (size_t)T * sizeof(K) + 16;
   static constexpr size_t vbuf_bytes = PAIRS ? (size_t)T * 4 + 16 : 0;
-  static constexpr size_t whist_bytes = (size_t)NW * kRadix * 8;  // [NW][256] lane masks, then [NW][256] counts
+  static constexpr size_t whist_bytes = (size_t)NW * kRadix * 4;  // [NW][256] digit counts
   static constexpr size_t small_bytes = 2 * kRadix * 4 + 64 * 4 + 2 * 8;
   static constexpr size_t smem_bytes = kbuf_bytes + vbuf_bytes + whist_bytes + small_bytes;
 };
@@ -138,35 +148,79 @@ struct TileCtx {
   const uint32_t* bin_offsets;  // this place's 256 bin offsets (segment-relative)
 };
 
-// Warp-level multi-split ranking of one 32-key batch (step 4). Returns the
-// key's rank among the keys of the same digit in this warp's part of the tile.
-// msk / cnt: this warp's 256 lane-mask words and 256 running digit counts
-// (separate 32-bit arrays, so random digits spread over all 32 banks).
+__device__ __forceinline__ uint32_t lanemask_ge() {
+  uint32_t m;
+  asm("mov.u32 %0, %%lanemask_ge;" : "=r"(m));
+  return m;
+}
+
+// Warp-level multi-split ranking of one 32-key batch with ballots. Returns the
+// value the warp's running counter of the key's digit has just before the key
+// (its rank among the warp's equal digits, or its local position when the
+// counters start at local positions). cnt: this warp's 256 running counters.
 template <bool FULL, int RB = kRadixBits>
-__device__ __forceinline__ uint32_t wlms_rank(uint32_t* msk, uint32_t* cnt, uint32_t d, bool valid, uint32_t lane_bit,
-                                              bool smask) {
-  // the running count first: its shared-memory round trip overlaps the
-  // search for peers (the previous batch's update is already visible)
+__device__ __forceinline__ uint32_t rank_ballot(uint32_t* cnt, uint32_t d, bool valid) {
+  // the running count first: its shared-memory round trip overlaps the votes
+  // (the previous batch's update is already visible)
   const uint32_t old = valid ? cnt[d] : 0u;
-  uint32_t peers;
-  if (smask) {
-    // every lane ORs its bit into its digit's mask word; OR commutes, so the
-    // mask read back is exactly the lanes sharing the digit
-    if (valid) atomicOr(msk + d, lane_bit);
-    __syncwarp();
-    peers = valid ? msk[d] : 0u;
-  } else {
-    const uint32_t valid_mask = FULL ? 0xFFFFFFFFu : __ballot_sync(0xFFFFFFFFu, valid);
-    peers = digit_peers<RB>(d, valid, valid_mask);
-  }
+  const uint32_t valid_mask = FULL ? 0xFFFFFFFFu : __ballot_sync(0xFFFFFFFFu, valid);
+  const uint32_t peers = digit_peers<RB>(d, valid, valid_mask);
   const uint32_t below = __popc(peers & lanemask_lt());
   __syncwarp();
-  if (valid && below == 0) {
-    if (smask) msk[d] = 0u;
-    cnt[d] = old + __popc(peers);
-  }
+  if (valid && below == 0) cnt[d] = old + __popc(peers);
   __syncwarp();
   return old + below;
+}
+
+// The same for U batches with counting atomics. Every lane adds 1 to the low
+// half of its digit's counter and its lane number to the high half; the old
+// low half is then the key's rank if lanes sharing a digit were served in lane
+// order. That order is not defined, so it is checked: after a warp barrier
+// every lane reads its counter again, and the difference to its old value
+// holds how many sharers were served from this lane on and the sum of their
+// lane numbers. A lane that finds itself last, or followed by exactly one
+// sharer in a higher lane, is in order; the digits of all other lanes (three
+// or more sharers, or a pair served in reverse) are settled one by one with a
+// vote on the digit and the lane numbers. Uniform 8-bit digits need that in
+// one batch of thirteen when pairs are served in lane order, and in most
+// batches otherwise. The batches' atomics and reads do not depend on the
+// checks, so a chunk's shared-memory round trips overlap. The running counts
+// stay below 2^16 (a tile's keys), so the halves do not mix.
+//
+// The ranking is bound by the L1 data pipe, which moves one wavefront a cycle
+// and takes 3.4 for 32 random digits' counters. A batch costs two such
+// accesses here, and no chain runs from one batch to the next; lane masks in
+// shared memory (OR, read, clear) beside a counter's read and update cost five
+// and a chain of round trips. The keys-only kernel went from 29.9 to 23.5
+// wavefronts and from 78 to 66 instructions per 32 keys, and a 2^28 pass of
+// the same 6144-key tiles from 0.944 to 0.838 ms (pairs 1.232 to 1.128).
+// Settling every shared digit with votes, without the lane sums, took 1.04 ms.
+template <bool FULL, int U>
+__device__ __forceinline__ void rank_atomic(uint32_t* cnt, const uint32_t (&d)[U], const bool (&valid)[U],
+                                            uint32_t (&rank)[U]) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t inc = (lane << 16) + 1u;
+  uint32_t old[U], after[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    old[u] = (FULL || valid[u]) ? atomicAdd(cnt + d[u], inc) : 0u;
+    __syncwarp();
+    after[u] = (FULL || valid[u]) ? *const_cast<volatile uint32_t*>(cnt + d[u]) : inc;
+    __syncwarp();
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    rank[u] = old[u] & 0xFFFFu;
+    const uint32_t later = after[u] - old[u] - inc;  // sharers served after this lane: count, sum of lanes
+    uint32_t open = __ballot_sync(0xFFFFFFFFu, (later & 0xFFFEu) != 0u || later - 1u < (lane << 16));
+    while (open) {
+      const uint32_t dl = __shfl_sync(0xFFFFFFFFu, d[u], 31 - __clz(open));
+      const bool same = d[u] == dl && (FULL || valid[u]);
+      const uint32_t peers = __ballot_sync(0xFFFFFFFFu, same);
+      if (same) rank[u] = (after[u] & 0xFFFFu) - __popc(peers & lanemask_ge());
+      open &= ~peers;
+    }
+  }
 }
 
 // Decoupled look-back of one digit in rounds: issue() reads the counters of
@@ -281,11 +335,10 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
 
   K* kt = reinterpret_cast<K*>(smem) + c.koff;
   uint32_t* vt = reinterpret_cast<uint32_t*>(smem + C::kbuf_bytes) + c.voff;
-  // [NW][256] lane masks of the current batch, then [NW][256] digit counts
-  // (turned into running local positions before the ranking)
-  uint32_t* whist = reinterpret_cast<uint32_t*>(smem + C::kbuf_bytes + C::vbuf_bytes);
-  uint32_t* wcnt = whist + NW * kRadix;
-  uint32_t* dstart = whist + 2 * NW * kRadix;  // [256] tile-local start of each digit's bin
+  // [NW][256] digit counts (turned into running local positions before the
+  // ranking)
+  uint32_t* wcnt = reinterpret_cast<uint32_t*>(smem + C::kbuf_bytes + C::vbuf_bytes);
+  uint32_t* dstart = wcnt + NW * kRadix;       // [256] tile-local start of each digit's bin
   uint32_t* gbase = dstart + kRadix;           // [256] segment index of local position 0 of each bin
   uint32_t* misc = gbase + kRadix;             // [64] scan scratch
   uint64_t* mbar = reinterpret_cast<uint64_t*>(misc + 64);
@@ -304,14 +357,10 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   const bool publish = (int64_t)tile != a.fault_tile;
   const bool chain_head = tile == c.chain_first;
 
-  // this warp's lane masks and counts start at zero
-  uint32_t* wmsk = whist + warp * kRadix;
+  // this warp's counts start at zero
   uint32_t* wc = wcnt + warp * kRadix;
 #pragma unroll
-  for (int i = lane; i < R; i += 32) {
-    wmsk[i] = 0u;
-    wc[i] = 0u;
-  }
+  for (int i = lane; i < R; i += 32) wc[i] = 0u;
 
   if (c.bulk) {
     if (!mbar_wait_bounded(&mbar[0], 0, kBulkWaitLimit)) atomicOr(a.error, kErrTimeout);
@@ -398,21 +447,34 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
     //     (every key is in registers since the barrier above); for pairs the
     //     positions are kept, two 16-bit positions per register
     uint32_t pos2[PAIRS ? IPT / 2 + 1 : 1];
-    const uint32_t lane_bit = 1u << lane;
+    constexpr int U = RANK == kRankBallot ? 1 : rank_chunk(PAIRS, IPT);
+    static_assert(IPT % U == 0 && kRoundEvery % U == 0, "whole chunks of batches");
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      const bool valid = FULL || wbase + i * 32 < count;
-      const bool smask = RANK == kRankHybrid && hybrid_uses_masks(i);
-      const uint32_t p = wlms_rank<FULL, RB>(wmsk, wc, digit_of(key[i], shift, mask, dxor), valid, lane_bit, smask);
-      if (valid) kt[p] = key[i];
-      if (PAIRS) {
-        if (i & 1)
-          pos2[i / 2] |= p << 16;
-        else
-          pos2[i / 2] = p;
+    for (int i0 = 0; i0 < IPT; i0 += U) {
+      uint32_t d[U], p[U];
+      bool valid[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        valid[u] = FULL || wbase + (i0 + u) * 32 < count;
+        d[u] = digit_of(key[i0 + u], shift, mask, dxor);
+      }
+      if constexpr (RANK == kRankBallot)
+        p[0] = rank_ballot<FULL, RB>(wc, d[0], valid[0]);
+      else
+        rank_atomic<FULL, U>(wc, d, valid, p);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u;
+        if (valid[u]) kt[p[u]] = key[i];
+        if (PAIRS) {
+          if (i & 1)
+            pos2[i / 2] |= p[u] << 16;
+          else
+            pos2[i / 2] = p[u];
+        }
       }
       // a look-back round: fold in the last one's reads, send the next
-      if (i % kRoundEvery == kRoundEvery - 1 && i + 1 < IPT && walker) {
+      if ((i0 + U) % kRoundEvery == 0 && i0 + U < IPT && walker) {
         if (issued) lb.consume();
         issued = !lb.done;
         if (issued) lb.issue(a.status, c.chain_first, tid);
@@ -498,7 +560,7 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
   K* kbuf = reinterpret_cast<K*>(smem);
   uint32_t* vbuf = reinterpret_cast<uint32_t*>(smem + C::kbuf_bytes);
   uint32_t* whist = reinterpret_cast<uint32_t*>(smem + C::kbuf_bytes + C::vbuf_bytes);
-  uint32_t* misc = whist + 2 * NW * kRadix + 2 * kRadix;
+  uint32_t* misc = whist + NW * kRadix + 2 * kRadix;
   uint64_t* mbar = reinterpret_cast<uint64_t*>(misc + 64);
   __shared__ TileCtx s_ctx;
   const int tid = threadIdx.x;
@@ -579,8 +641,8 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
   }
 
   // adaptive ranking: one uniform branch per tile between two whole bodies
-  // (ballots for a skewed place, the hybrid otherwise)
-  constexpr int R0 = RANK == kRankAdaptive ? kRankHybrid : RANK;
+  // (ballots for a skewed place, counting atomics otherwise)
+  constexpr int R0 = RANK == kRankAdaptive ? kRankAtomic : RANK;
   const bool ballots = RANK == kRankAdaptive && c.skewed;
   if (c.count == (uint32_t)T) {
     if (ballots)

@@ -83,8 +83,8 @@ struct WsConfig {
   static constexpr size_t stage_v = al(stage_k + (size_t)T * sizeof(K) + 16);
   static constexpr size_t sorted = al(stage_v + (PAIRS ? (size_t)T * 4 + 16 : 0));
   static constexpr size_t sorted_bytes = al((size_t)T * (sizeof(K) + kVB));  // keys then values
-  static constexpr size_t tables = sorted + 2 * sorted_bytes;              // [NR][256] lane masks, [NR][256] counts
-  static constexpr size_t meta = tables + (size_t)NR * kRadix * 8;         // per sorted buffer: dstart[256], count[256]
+  static constexpr size_t tables = sorted + 2 * sorted_bytes;              // [NR][256] digit counts
+  static constexpr size_t meta = tables + (size_t)NR * kRadix * 4;         // per sorted buffer: dstart[256], count[256]
   static constexpr size_t gbase = meta + 2 * 2 * kRadix * 4;               // writers: [256]
   static constexpr size_t scan = gbase + kRadix * 4;                       // rankers' scan scratch [32]
   static constexpr size_t ctx = scan + 32 * 4;                             // WsTile: staging, sorted 0, sorted 1
@@ -248,9 +248,7 @@ __device__ __forceinline__ void ws_rank_tile(const PassArgs& a, unsigned char* s
   const int shift = a.shift;
   const uint32_t mask = a.mask, dxor = a.digit_xor;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::bars);
-  uint32_t* tables = reinterpret_cast<uint32_t*>(smem + C::tables);
-  uint32_t* wmsk_all = tables;                  // [NR][256]
-  uint32_t* wcnt_all = tables + NR * kRadix;    // [NR][256]
+  uint32_t* wcnt_all = reinterpret_cast<uint32_t*>(smem + C::tables);  // [NR][256]
   uint32_t* meta = reinterpret_cast<uint32_t*>(smem + C::meta) + b * 2 * kRadix;
   uint32_t* dstart = meta;                      // [256]
   uint32_t* dcount = meta + kRadix;             // [256]
@@ -337,20 +335,32 @@ __device__ __forceinline__ void ws_rank_tile(const PassArgs& a, unsigned char* s
     }
   } else {
     // 2. warp-level multi-split ranking (Section 3, WLMS); RANK is the
-    //    ballot or the hybrid method here
-    uint32_t* wmsk = wmsk_all + warp * kRadix;
+    //    ballot or the atomic method here
     uint32_t* wc = wcnt_all + warp * kRadix;
     uint32_t rank2[IPT / 2 + 1];
-    const uint32_t lane_bit = 1u << lane;
+    constexpr int U = RANK == kRankBallot ? 1 : rank_chunk(PAIRS, IPT);
+    static_assert(IPT % U == 0, "whole chunks of batches");
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      const bool valid = FULL || wbase + i * 32 < count;
-      const bool smask = RANK == kRankHybrid && hybrid_uses_masks(i);
-      const uint32_t r = wlms_rank<FULL>(wmsk, wc, digit_of(key[i], shift, mask, dxor), valid, lane_bit, smask);
-      if (i & 1)
-        rank2[i / 2] |= r << 16;
+    for (int i0 = 0; i0 < IPT; i0 += U) {
+      uint32_t d[U], r[U];
+      bool valid[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        valid[u] = FULL || wbase + (i0 + u) * 32 < count;
+        d[u] = digit_of(key[i0 + u], shift, mask, dxor);
+      }
+      if constexpr (RANK == kRankBallot)
+        r[0] = rank_ballot<FULL>(wc, d[0], valid[0]);
       else
-        rank2[i / 2] = r;
+        rank_atomic<FULL, U>(wc, d, valid, r);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u;
+        if (i & 1)
+          rank2[i / 2] |= r[u] << 16;
+        else
+          rank2[i / 2] = r[u];
+      }
     }
     named_bar_sync(kBarRankers, NRT);
 
@@ -359,7 +369,7 @@ __device__ __forceinline__ void ws_rank_tile(const PassArgs& a, unsigned char* s
     uint32_t c = 0;
     if (rt < kRadix) {
 #pragma unroll
-      for (int w = 0; w < NR; ++w) c += wcnt_all[w * kRadix + rt];
+      for (int w = 0; w < NR; ++w) c += wcnt_all[w * kRadix + rt] & 0xFFFFu;  // (atomic ranking uses the high halves)
       if (publish) st_relaxed_gpu(status + rt, ((head ? kFlagGlobal : kFlagLocal) << kStatusShift) | c);
     }
     const uint32_t excl = ranker_exclusive_sum<NRT>(rt < kRadix ? c : 0u, scan);
@@ -367,7 +377,7 @@ __device__ __forceinline__ void ws_rank_tile(const PassArgs& a, unsigned char* s
       uint32_t run = excl;
 #pragma unroll
       for (int w = 0; w < NR; ++w) {
-        const uint32_t cw = wcnt_all[w * kRadix + rt];
+        const uint32_t cw = wcnt_all[w * kRadix + rt] & 0xFFFFu;
         wcnt_all[w * kRadix + rt] = run;
         run += cw;
       }
@@ -414,7 +424,7 @@ __device__ void ws_rankers(const PassArgs& a, unsigned char* smem) {
   const int rt = threadIdx.x;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::bars);
   const WsTile* sctx = reinterpret_cast<const WsTile*>(smem + C::ctx);
-  constexpr int R1 = RANK == kRankBallot ? kRankBallot : kRankHybrid;
+  constexpr int R1 = RANK == kRankBallot ? kRankBallot : kRankAtomic;
   const bool ballots = RANK == kRankBallot || (RANK == kRankAdaptive && a.skew_flags && *a.skew_flags);
 
   // thread 0 stages the first tile and takes the id of the second
@@ -440,7 +450,7 @@ __device__ void ws_rankers(const PassArgs& a, unsigned char* smem) {
       return;
     }
     // one uniform branch per tile between whole tile bodies: ballots only
-    // (a skewed place, or the ballot variant) or the hybrid
+    // (a skewed place, or the ballot variant) or the counting atomics
     bool stop = false;
     if (t.count == (uint32_t)C::T) {
       if (ballots)
@@ -573,10 +583,10 @@ __global__ void __launch_bounds__(WsConfig<KBITS, PAIRS>::NT, 1) binning_ws_kern
     mbar_init(bars + 6, 1);
     fence_mbar_init();
   }
-  // lane-mask and count tables start at zero (ranking leaves the masks at
-  // zero; each warp zeroes its counts after its reorganisation)
+  // the count tables start at zero (each warp zeroes its own again after its
+  // reorganisation)
   uint32_t* tables = reinterpret_cast<uint32_t*>(smem + C::tables);
-  for (int i = tid; i < C::NR * kRadix * 2; i += C::NT) tables[i] = 0u;
+  for (int i = tid; i < C::NR * kRadix; i += C::NT) tables[i] = 0u;
   __syncthreads();
   if (warp < C::NR)
     ws_rankers<KBITS, PAIRS, RANK, FLIP>(a, smem);
@@ -652,7 +662,7 @@ template <int KBITS, bool PAIRS, int FLIP, bool SEG>
 cudaError_t launch_binning_flip(const PassArgs& a, cudaStream_t s, int cfg, int rank) {
   switch (rank) {
     case kRankAdaptive: return launch_binning_flip_rank<KBITS, PAIRS, FLIP, kRankAdaptive, SEG>(a, s, cfg);
-    case kRankHybrid: return launch_binning_flip_rank<KBITS, PAIRS, FLIP, kRankHybrid, SEG>(a, s, cfg);
+    case kRankAtomic: return launch_binning_flip_rank<KBITS, PAIRS, FLIP, kRankAtomic, SEG>(a, s, cfg);
     default: return launch_binning_flip_rank<KBITS, PAIRS, FLIP, kRankBallot, SEG>(a, s, cfg);
   }
 }
