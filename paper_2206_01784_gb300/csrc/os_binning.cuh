@@ -46,8 +46,12 @@
 //
 // In segmented mode (os_sort_batch) every segment is a sort of its own: its
 // tiles form one look-back chain that starts at the segment's first tile, and
-// it has its own bin offsets. Full tiles take a branch-light path with no
-// per-key bounds checks; only a ragged tile checks every index.
+// it has its own bin offsets.
+//
+// There are no per-key bounds checks: a chain's ragged last tile is filled up
+// with keys that sort behind it and are never stored. A second body for it
+// would be fetched cold by one block at the very end of every pass, which
+// costs a pass about 25 us (8.0M u32 pairs: 78 us a pass, 2^23 pairs: 49).
 #pragma once
 
 #include "os_common.cuh"
@@ -67,13 +71,15 @@ namespace onesweep {
 // 0.730, 512 x 24 x 2 1.34 / 0.742, 256 x 40 x 2 1.07 / 0.799, 512 x 32 x 1
 // 1.20 / 0.868; at 2^27 u64: 256 x 12 x 3 0.905 / 0.741, 256 x 16 x 3 0.788 /
 // 0.630, 256 x 20 x 3 0.714 / 0.566, 256 x 24 x 2 0.765 / 0.606. The smaller
-// tiles were not faster at any size from 2^21 to 2^25 either.
+// tiles are faster only where the largest one makes little more than one wave
+// of blocks (4.2M u32 pairs: 124 us a sort with geometry 1 against 133, 6.5M
+// 176 against 174).
 template <int KBITS, int CFG> struct TileShape;
 template <> struct TileShape<32, 0> { static constexpr int NT = 256, IPT = 32, MINB = 3; };
-template <> struct TileShape<32, 1> { static constexpr int NT = 256, IPT = 20, MINB = 3; };
+template <> struct TileShape<32, 1> { static constexpr int NT = 256, IPT = 24, MINB = 3; };
 template <> struct TileShape<32, 2> { static constexpr int NT = 256, IPT = 16, MINB = 4; };
 template <> struct TileShape<64, 0> { static constexpr int NT = 256, IPT = 20, MINB = 3; };
-template <> struct TileShape<64, 1> { static constexpr int NT = 256, IPT = 10, MINB = 3; };
+template <> struct TileShape<64, 1> { static constexpr int NT = 256, IPT = 16, MINB = 3; };
 template <> struct TileShape<64, 2> { static constexpr int NT = 256, IPT = 8, MINB = 4; };
 
 // Digit-ranking variants of step 6. Two methods find a key's rank among the
@@ -325,7 +331,7 @@ constexpr uint32_t kPrefetchTiles = 48;
 #endif
 constexpr int kRoundEvery = OS_ROUND_EVERY;
 
-template <int KBITS, bool PAIRS, int CFG, int RANK, int FLIP, bool FULL, int RB>
+template <int KBITS, bool PAIRS, int CFG, int RANK, int FLIP, int RB>
 __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* smem, const TileCtx& c) {
   using C = BinningConfig<KBITS, PAIRS, CFG>;
   using K = typename C::K;
@@ -347,7 +353,8 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   const int shift = a.shift;
   const uint32_t mask = a.mask;
   const uint32_t dxor = a.digit_xor;
-  const uint32_t tile = c.tile, count = c.count;
+  const uint32_t tile = c.tile;
+  const uint32_t pads = (uint32_t)C::T - c.count;  // of a ragged tile
 
   // the next pass's status counters of this tile start at N
   if (a.status_clear && tid < kRadix)
@@ -367,6 +374,16 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   } else {
     __syncthreads();
   }
+  if (pads) {
+    // a ragged tile (the last of its chain) is filled up with keys of the
+    // pass's highest digit: they sort behind every key of the tile, are left
+    // out of the published counts, and their places lie past the chain's end,
+    // where the scatter's range check drops them
+    const K ordered = (K)(mask ^ dxor) << shift;
+    const K pad = (FLIP & 1) ? flip_from_ordered(ordered) : ordered;
+    for (uint32_t i = c.count + tid; i < (uint32_t)C::T; i += NT) kt[i] = pad;
+    __syncthreads();
+  }
   __syncwarp();
 
   // keys of this thread: warp-striped, batch i of warp w covers tile positions
@@ -374,15 +391,11 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   K key[IPT];
   const uint32_t wbase = (uint32_t)warp * IPT * 32 + lane;
 #pragma unroll
-  for (int i = 0; i < IPT; ++i) {
-    const uint32_t idx = wbase + i * 32;
-    key[i] = load_transform<FLIP>((FULL || idx < count) ? kt[idx] : K(0));
-  }
+  for (int i = 0; i < IPT; ++i) key[i] = load_transform<FLIP>(kt[wbase + i * 32]);
 
   // 3. early counts: each warp's digit histogram of its part of the tile
 #pragma unroll
-  for (int i = 0; i < IPT; ++i)
-    if (FULL || wbase + i * 32 < count) atomicAdd(wc + digit_of(key[i], shift, mask, dxor), 1u);
+  for (int i = 0; i < IPT; ++i) atomicAdd(wc + digit_of(key[i], shift, mask, dxor), 1u);
   const uint32_t d0 = digit_of(load_transform<FLIP>(kt[0]), shift, mask, dxor);
   if (tid == 0) misc[NW] = 0u;  // set below by the digit that holds every key, if one does
   __syncthreads();
@@ -390,10 +403,12 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   // 4. tile digit counts: publish L now, and start the look-back (step 6),
   //    whose rounds then ride along the ranking; a tile whose keys share one
   //    digit skips ranking and reorganisation (homogeneous-tile short-circuit)
-  uint32_t digit_count = 0;  // thread d < 256: keys of digit d in this tile
+  uint32_t filled = 0;       // thread d < 256: keys of digit d in this tile, the pads included ...
+  uint32_t digit_count = 0;  // ... and without
   if (tid < R) {
 #pragma unroll
-    for (int w = 0; w < NW; ++w) digit_count += wcnt[w * kRadix + tid];
+    for (int w = 0; w < NW; ++w) filled += wcnt[w * kRadix + tid];
+    digit_count = filled - ((uint32_t)tid == mask ? pads : 0u);
     if (publish)
       st_relaxed_gpu(status + tid, ((chain_head ? kFlagGlobal : kFlagLocal) << kStatusShift) | digit_count);
   }
@@ -410,14 +425,14 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   // block scan of the counts (a warp scan, one barrier, the lower warps'
   // totals), which also tells whether every key has the same digit
   static_assert(NW < 64, "scan scratch");
-  uint32_t incl = tid < R ? digit_count : 0u;
+  uint32_t incl = filled;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += y;
   }
   if (lane == 31) misc[warp] = incl;
-  if (tid < R && digit_count == count) misc[NW] = 1u;
+  if (filled == (uint32_t)C::T) misc[NW] = 1u;
   __syncthreads();
   const bool homogeneous = misc[NW] != 0u;
 
@@ -427,7 +442,7 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   } else {
     // 5. tile-local bin starts, and each warp's counters set to where its
     //    first key of each digit goes
-    uint32_t excl = incl - (tid < R ? digit_count : 0u);
+    uint32_t excl = incl - filled;
     for (int w = 0; w < NW; ++w)
       if (w < warp) excl += misc[w];
     if (tid < R) {
@@ -452,20 +467,17 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
 #pragma unroll
     for (int i0 = 0; i0 < IPT; i0 += U) {
       uint32_t d[U], p[U];
-      bool valid[U];
+      const bool valid[U] = {};
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        valid[u] = FULL || wbase + (i0 + u) * 32 < count;
-        d[u] = digit_of(key[i0 + u], shift, mask, dxor);
-      }
+      for (int u = 0; u < U; ++u) d[u] = digit_of(key[i0 + u], shift, mask, dxor);
       if constexpr (RANK == kRankBallot)
-        p[0] = rank_ballot<FULL, RB>(wc, d[0], valid[0]);
+        p[0] = rank_ballot<true, RB>(wc, d[0], true);
       else
-        rank_atomic<FULL, U>(wc, d, valid, p);
+        rank_atomic<true, U>(wc, d, valid, p);  // (every lane is valid)
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u;
-        if (valid[u]) kt[p[u]] = key[i];
+        kt[p[u]] = key[i];
         if (PAIRS) {
           if (i & 1)
             pos2[i / 2] |= p[u] << 16;
@@ -485,14 +497,10 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
       if (c.bulk && !mbar_wait_bounded(&mbar[1], 0, kBulkWaitLimit)) atomicOr(a.error, kErrTimeout);
       uint32_t val[IPT];
 #pragma unroll
-      for (int i = 0; i < IPT; ++i) {
-        const uint32_t idx = wbase + i * 32;
-        val[i] = (FULL || idx < count) ? vt[idx] : 0u;
-      }
+      for (int i = 0; i < IPT; ++i) val[i] = vt[wbase + i * 32];
       __syncthreads();
 #pragma unroll
-      for (int i = 0; i < IPT; ++i)
-        if (FULL || wbase + i * 32 < count) vt[(i & 1) ? (pos2[i / 2] >> 16) : (pos2[i / 2] & 0xFFFFu)] = val[i];
+      for (int i = 0; i < IPT; ++i) vt[(i & 1) ? (pos2[i / 2] >> 16) : (pos2[i / 2] & 0xFFFFu)] = val[i];
     }
   }
 
@@ -521,26 +529,22 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
 #pragma unroll 4
     for (int i = 0; i < IPT; ++i) {
       const uint32_t j = i * NT + tid;
-      if (FULL || j < count) {
-        const K k = store_transform<FLIP>(load_transform<FLIP>(kt[j]));
-        const uint32_t g = g0 + j;
-        if (g < out_len) {
-          keys_out[g] = k;
-          if (PAIRS) vals_out[g] = vt[j];
-        }
+      const K k = store_transform<FLIP>(load_transform<FLIP>(kt[j]));
+      const uint32_t g = g0 + j;
+      if (g < out_len) {
+        keys_out[g] = k;
+        if (PAIRS) vals_out[g] = vt[j];
       }
     }
   } else {
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
       const uint32_t j = i * NT + tid;
-      if (FULL || j < count) {
-        const K k = kt[j];
-        const uint32_t g = gbase[digit_of(k, shift, mask, dxor)] + j;
-        if (g < out_len) {
-          keys_out[g] = store_transform<FLIP>(k);
-          if (PAIRS) vals_out[g] = vt[j];
-        }
+      const K k = kt[j];
+      const uint32_t g = gbase[digit_of(k, shift, mask, dxor)] + j;
+      if (g < out_len) {
+        keys_out[g] = store_transform<FLIP>(k);
+        if (PAIRS) vals_out[g] = vt[j];
       }
     }
   }
@@ -644,17 +648,10 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
   // (ballots for a skewed place, counting atomics otherwise)
   constexpr int R0 = RANK == kRankAdaptive ? kRankAtomic : RANK;
   const bool ballots = RANK == kRankAdaptive && c.skewed;
-  if (c.count == (uint32_t)T) {
-    if (ballots)
-      binning_tile<KBITS, PAIRS, CFG, kRankBallot, FLIP, true, RB>(a, smem, c);
-    else
-      binning_tile<KBITS, PAIRS, CFG, R0, FLIP, true, RB>(a, smem, c);
-  } else {
-    if (ballots)
-      binning_tile<KBITS, PAIRS, CFG, kRankBallot, FLIP, false, RB>(a, smem, c);
-    else
-      binning_tile<KBITS, PAIRS, CFG, R0, FLIP, false, RB>(a, smem, c);
-  }
+  if (ballots)
+    binning_tile<KBITS, PAIRS, CFG, kRankBallot, FLIP, RB>(a, smem, c);
+  else
+    binning_tile<KBITS, PAIRS, CFG, R0, FLIP, RB>(a, smem, c);
 }
 
 }  // namespace onesweep
