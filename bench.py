@@ -294,8 +294,9 @@ def measure_config(torch, osw, workload, np, dev, key_type: str, log2n: int, pai
     if not bool((ok64[1:] >= ok64[:-1]).all().item()):
         raise RuntimeError("configuration output not sorted")
     peak, _ = hbm_peak()
-    bin_ms = statistics.mean([m for k, _, m in recs if k == 1])
-    hist_ms = statistics.mean([m for k, _, m in recs if k == 0])
+    # (a sort small enough for one launch, kernel 4, has no passes of its own)
+    bin_ms = statistics.mean([m for k, _, m in recs if k == 1] or [m / places for k, _, m in recs if k == 4])
+    hist_ms = statistics.mean([m for k, _, m in recs if k == 0] or [0.0])
     per_pass = n * 2 * (kbytes + (4 if pairs else 0))
     step_bytes = n * kbytes + places * per_pass
     return {"workload": workload_name(n, dist, seed, pairs, key_type), "keys": n, "places": places,
@@ -607,7 +608,8 @@ def main():
 
     # roofline of the dominant kernel (the binning pass)
     peak, peak_kind = hbm_peak()
-    bin_ms = [ms for k, _, ms in recs if k == 1]
+    # (a sort small enough for one launch, kernel 4, has no passes of its own)
+    bin_ms = [ms for k, _, ms in recs if k == 1] or [ms / lay.num_places for k, _, ms in recs if k == 4]
     hist_ms = [ms for k, _, ms in recs if k == 0]
     bin_avg = statistics.mean(bin_ms)
     bytes_per_pass = n * 2 * (kbytes + (4 if pairs else 0))

@@ -92,7 +92,11 @@ typedef enum {
     OS_ERR_SCRATCH_LIMIT = 6 /* os_sort_noalloc: the sort needs more than its fixed scratch */
 } os_status;
 
-/* Where the parts of a sort's workspace sit (byte offsets from ws). */
+/*
+ * Where the parts of a sort's workspace sit (byte offsets from ws). A sort
+ * that runs as one launch (below) uses the status word at ws and the space of
+ * the others as it needs, and leaves no histograms or counters there.
+ */
 typedef struct {
     size_t total_bytes;        /* what os_sort_workspace_bytes() returns */
     size_t status_offset[2];   /* the two status-counter slabs (pass i uses slab i % 2) */
@@ -117,6 +121,15 @@ OS_API size_t os_sort_workspace_bytes(int key_type, uint64_t n, int value_bytes,
 /* Fills *layout for the same arguments. Returns OS_OK or OS_ERR_INVALID_ARG. */
 OS_API int os_sort_workspace_layout(int key_type, uint64_t n, int value_bytes, int begin_bit, int end_bit,
                              os_workspace_layout *layout);
+
+/*
+ * Sorts of up to about two million keys (12288 32-bit or 8192 64-bit keys per
+ * SM of the device) run as one launch that keeps the keys on the chip between
+ * passes, unless the caller names a tile variant or a digit width other than 8,
+ * the bit range is a single place of more than 4096 keys, or the blocks cannot
+ * all be resident at once; the result is the same. On up to 16384 keys the
+ * launch is one block or one cluster; above, a cooperative grid.
+ */
 
 /*
  * Sorts n keys (Section 3, all three phases). keys_in: n keys (device);
@@ -267,7 +280,9 @@ OS_API int os_sort_noalloc(int key_type, const void *keys_in, void *keys_out, co
                            const void **scratch_out);
 
 /*
- * Tile geometry of the digit-binning kernel (tuning, not part of the method).
+ * Tile geometry of the digit-binning kernel (tuning, not part of the method),
+ * for the sorts that run it: a sort small enough for one launch uses the
+ * geometry only when the call names it (os_sort_options).
  * There are os_num_tile_configs() geometries per key width and payload
  * (keys only: value_bytes 0, pairs: 4); os_tile_config_keys() gives the keys
  * per tile of one (0 for invalid arguments). os_set_tile_config() selects the
@@ -318,8 +333,9 @@ OS_API int os_get_radix_bits_bucket(int key_bits, int value_bytes, int bucket);
  */
 typedef struct {
     int kernel;   /* 0 = histogram (phases 1-2), 1 = digit binning (phase 3),
-                     2 = batch plan, 3 = batch one-block sort of small segments */
-    int pass;     /* digit place of a binning launch, -1 for the histogram */
+                     2 = batch plan, 3 = batch one-block sort of small segments,
+                     4 = a whole small sort */
+    int pass;     /* digit place of a binning launch, -1 otherwise */
     float ms;     /* device time between the pair of events */
 } os_launch_time;
 

@@ -384,6 +384,53 @@ int run_histogram(const Plan& plan, int key_type, const void* keys, uint64_t n, 
   return e == cudaSuccess ? OS_OK : OS_ERR_CUDA;
 }
 
+// The whole sort in one launch, when it is small enough and nothing asks for
+// the pass-by-pass kernels (a named variant or digit width, a test hook).
+// Returns whether it was launched; *rc is then its status.
+bool run_small(const Plan& plan, int key_type, const void* keys_in, void* keys_out, const uint32_t* vals_in,
+               uint32_t* vals_out, uint64_t n, int begin_bit, int end_bit, char* w, cudaStream_t s, int* rc) {
+  if (plan.radix_bits != kRadixBits || plan.strips != 1 || plan.fault_tile >= 0) return false;
+  const int form = small_form(plan.key_bits, plan.pairs, n, device_sm_count());
+  if (form == 0) return false;
+  const uint32_t blocks = small_blocks(form, n);
+  const os_workspace_layout& L = plan.layout;
+  SmallArgs a{};
+  if (blocks > 1 && plan.places < 2) return false;  // one pass: nothing to gain
+  if (small_needs_matrices(form)) {
+    // the count matrices take the place of the status slabs
+    if ((size_t)blocks * 32 * sizeof(uint4) > L.status_offset[1] - L.status_offset[0]) return false;
+    a.alt_keys = w + L.alt_keys_offset;
+    a.alt_vals = reinterpret_cast<uint32_t*>(w + L.alt_values_offset);
+    a.counts_even = reinterpret_cast<uint4*>(w + L.status_offset[0]);
+    a.counts_odd = reinterpret_cast<uint4*>(w + L.status_offset[1]);
+  }
+  a.keys_in = keys_in;
+  a.keys_out = keys_out;
+  a.vals_in = vals_in;
+  a.vals_out = vals_out;
+  a.error = reinterpret_cast<uint32_t*>(w);
+  a.n = (uint32_t)n;
+  a.flip = is_float(key_type);
+  a.num_places = plan.places;
+  a.begin_bit = begin_bit;
+  a.end_bit = end_bit;
+  a.top_xor = signed_top_xor(key_type, begin_bit, end_bit);
+  a.descending = is_descending(key_type) ? 1u : 0u;
+  a.spin_limit = plan.spin_limit;
+  const int slot = prof_begin(4, -1, s);
+  const cudaError_t e = launch_small(plan.key_bits, plan.pairs, form, a, s);
+  prof_end(slot, s);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
+      e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration) {
+    // the blocks cannot all be resident (a context with fewer SMs at hand than
+    // the device has): pass by pass
+    (void)cudaGetLastError();
+    return false;
+  }
+  *rc = e == cudaSuccess ? OS_OK : OS_ERR_CUDA;
+  return true;
+}
+
 int run_sort(int key_type, const void* keys_in, void* keys_out, const uint32_t* vals_in, uint32_t* vals_out,
              uint64_t n, int begin_bit, int end_bit, void* ws, size_t ws_bytes, void* stream, int cfg_override = -1,
              int radix_bits = 0) {
@@ -426,6 +473,9 @@ int run_sort(int key_type, const void* keys_in, void* keys_out, const uint32_t* 
       return OS_ERR_CUDA;
     return OS_OK;
   }
+
+  if (cfg_override < 0 && run_small(plan, key_type, keys_in, keys_out, vals_in, vals_out, n, begin_bit, end_bit, w, s, &rc))
+    return rc;
 
   // zero: status word, done counter, histograms, this sort's tile counters
   const size_t zero_bytes = plan.counters + (size_t)plan.places * plan.strips * 4;

@@ -74,6 +74,34 @@ struct PassArgs {
   uint32_t digit_xor;            // signed keys, top place: invert the digit's high bit (else 0)
 };
 
+// A whole sort in one launch (os_small.cu).
+struct SmallArgs {
+  const void* keys_in;
+  void* keys_out;
+  const uint32_t* vals_in;   // null for keys only
+  uint32_t* vals_out;
+  void* alt_keys;            // n keys and values between two passes (more than one block only)
+  uint32_t* alt_vals;
+  uint4* counts_even;        // [32][blocks] exchanged digit counts of even / odd passes
+  uint4* counts_odd;
+  uint32_t* error;           // device status word
+  uint32_t n;
+  int flip;                  // float keys
+  int num_places;
+  int begin_bit;
+  int end_bit;
+  uint32_t top_xor;          // signed keys: high bit of the top place's digit inverted (else 0)
+  uint32_t descending;       // bin by the complemented digit of every place
+  uint32_t spin_limit;       // polls of one block's counts before giving up
+};
+
+// Form of the one-launch sort for n keys on a device of `sms` SMs; 0: none
+// (the array is too large for it). small_blocks: its blocks.
+int small_form(int key_bits, bool pairs, uint64_t n, int sms);
+uint32_t small_blocks(int form, uint64_t n);
+bool small_needs_matrices(int form);  // exchanges counts through SmallArgs::counts_*
+cudaError_t launch_small(int key_bits, bool pairs, int form, const SmallArgs& a, cudaStream_t s);
+
 // Segmented sort: the plan, per-segment histograms and the one-block sort of
 // small segments (os_batch.cu).
 struct BatchArgs {

@@ -1,0 +1,199 @@
+// One block's part of a sort whose keys stay on the chip (os_small.cu, and the
+// short segments of a batch in os_batch.cu): a stable digit-binning pass of up
+// to NT * IPT keys held in registers, into digit order in shared memory.
+#pragma once
+
+#include "os_binning.cuh"
+
+namespace onesweep {
+
+template <int KBITS, bool PAIRS, int NT_, int IPT_>
+struct SmallTile {
+  using K = typename KeyWord<KBITS>::type;
+  static constexpr int NT = NT_, IPT = IPT_, NW = NT / 32;
+  static constexpr int T = NT * IPT;        // keys per tile
+  static constexpr int Q = NT / kRadix;     // parts of 8 warps, whose counts of a digit one thread adds up
+  static constexpr int WPP = NW / Q;
+  // with few keys a thread, the first pass's values are loaded beside its keys:
+  // both come from DRAM, and there are registers for both
+  static constexpr bool kValuesFirst = IPT <= 4;
+  static_assert(NT % kRadix == 0 && Q <= 4 && T < (1 << 14), "tile shape (exchanged counts are 14 bits wide)");
+  // shared memory (bytes)
+  static constexpr size_t kbuf = 0;                                   // the tile in digit order
+  static constexpr size_t vbuf = kbuf + (size_t)T * sizeof(K);
+  static constexpr size_t wcnt = vbuf + (PAIRS ? (size_t)T * 4 : 0);  // [NW][256] running counts of each warp
+  static constexpr size_t psum = wcnt + (size_t)NW * kRadix * 4;      // [Q][256] digit counts of a part
+  static constexpr size_t gsum = psum + (size_t)Q * kRadix * 4;       // [Q][8] ... of 32 digits
+  static constexpr size_t smem_bytes = gsum + 32 * 4;
+
+  K key[IPT];
+  uint32_t val[PAIRS ? IPT : 1];
+  uint32_t count;   // keys in the tile
+  uint32_t wbase;   // tile position of this thread's first key
+  uint32_t total;   // threads 0..255, after bin(): the tile's count of digit tid ...
+  uint32_t excl;    // ... and of the digits below it
+
+  // This thread's keys: warp-striped, batch i of warp w covers positions
+  // [w*IPT*32 + i*32, +32), so batch order and lane order are tile order.
+  __device__ __forceinline__ void init(unsigned char* smem, uint32_t n) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    count = n;
+    wbase = (uint32_t)warp * IPT * 32 + lane;
+    clear_counts(smem);
+  }
+  __device__ __forceinline__ bool valid(int i) const { return wbase + i * 32 < count; }
+  __device__ __forceinline__ void clear_counts(unsigned char* smem) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint4* row = reinterpret_cast<uint4*>(smem + wcnt) + warp * (kRadix / 4);
+    row[lane] = make_uint4(0, 0, 0, 0);
+    row[lane + 32] = make_uint4(0, 0, 0, 0);
+  }
+  // kL2: read past L1 (which may hold what the buffer held two passes ago)
+  template <bool kL2 = false>
+  __device__ __forceinline__ void load_keys(const K* keys, int flip = 0) {
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) key[i] = !valid(i) ? K(0) : kL2 ? __ldcg(keys + wbase + i * 32) : keys[wbase + i * 32];
+    if (flip) {
+#pragma unroll
+      for (int i = 0; i < IPT; ++i) key[i] = flip_to_ordered(key[i]);
+    }
+  }
+  template <bool kL2 = false>
+  __device__ __forceinline__ void load_values(const uint32_t* vals) {
+    if (!PAIRS) return;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) val[i] = !valid(i) ? 0u : kL2 ? __ldcg(vals + wbase + i * 32) : vals[wbase + i * 32];
+  }
+
+  // One binning pass: on return kbuf (and vbuf) hold the tile in stable digit
+  // order, visible to the block, and total / excl are set. values() loads
+  // this thread's values: it is called once the keys are ranked, so the values
+  // take no registers before and their way here is covered by the scan.
+  // publish(total) is called by threads 0..255 as soon as the counts are known.
+  //
+  // Four barriers; what bounds a tile of a few thousand keys is their latency
+  // and that of the shared-memory round trips between them. So the scan over
+  // 256 digits takes no barrier of its own: each warp adds the sums of the
+  // lower groups of 32 digits itself (one load, one warp reduction).
+  template <typename Values, typename Publish>
+  __device__ __forceinline__ void bin(unsigned char* smem, int shift, uint32_t mask, uint32_t dxor, Values values,
+                                      Publish publish) {
+    constexpr int U = IPT % 4 == 0 ? 4 : 2;
+    K* kb = reinterpret_cast<K*>(smem + kbuf);
+    uint32_t* vb = reinterpret_cast<uint32_t*>(smem + vbuf);
+    uint32_t* wcnt_all = reinterpret_cast<uint32_t*>(smem + wcnt);
+    uint32_t* ps = reinterpret_cast<uint32_t*>(smem + psum);
+    uint32_t* gs = reinterpret_cast<uint32_t*>(smem + gsum);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t* wc = wcnt_all + warp * kRadix;
+
+    // rank each key among its warp's equal digits; a warp whose keys share one
+    // digit has nothing to rank (and its atomics would all meet in one counter)
+    uint32_t rank2[IPT / 2];  // two 16-bit ranks to a register
+    const uint32_t d0 = __shfl_sync(0xFFFFFFFFu, digit_of(key[0], shift, mask, dxor), 0);
+    bool differ = false;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) differ |= valid(i) && digit_of(key[i], shift, mask, dxor) != d0;
+    if (__any_sync(0xFFFFFFFFu, differ)) {
+#pragma unroll
+      for (int i0 = 0; i0 < IPT; i0 += U) {
+        uint32_t d[U], r[U];
+        bool v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          v[u] = valid(i0 + u);
+          d[u] = digit_of(key[i0 + u], shift, mask, dxor);
+        }
+        rank_atomic<false, U>(wc, d, v, r);
+#pragma unroll
+        for (int u = 0; u < U; u += 2) rank2[(i0 + u) / 2] = r[u] | r[u + 1] << 16;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < IPT; i += 2) rank2[i / 2] = (i * 32 + lane) | ((i + 1) * 32 + lane) << 16;
+      const uint32_t first = (uint32_t)warp * IPT * 32;
+      if (lane == 0 && count > first) wc[d0] = min((uint32_t)IPT * 32, count - first);
+    }
+    values();
+    __syncthreads();
+
+    // thread (q, d): digit d's counts in the 8 warps of part q
+    const int d = tid & (kRadix - 1), q = tid >> kRadixBits;
+    uint32_t part[WPP], sum = 0;
+#pragma unroll
+    for (int w = 0; w < WPP; ++w) {
+      part[w] = wcnt_all[(q * WPP + w) * kRadix + d] & 0xFFFFu;  // (the high halves hold lane sums)
+      sum += part[w];
+    }
+    if (Q > 1) ps[tid] = sum;
+    const uint32_t group = __reduce_add_sync(0xFFFFFFFFu, sum);
+    if (lane == 0) gs[warp] = group;  // warp = q * 8 + d / 32
+    __syncthreads();
+    uint32_t all = sum, lower = 0;  // digit d in the whole tile, and in the parts below q
+    if (Q > 1) {
+      all = 0;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const uint32_t p = ps[i * kRadix + d];
+        all += p;
+        if (i < q) lower += p;
+      }
+    }
+    if (tid < kRadix) publish(all);
+    const uint32_t below = __reduce_add_sync(0xFFFFFFFFu, lane < NW && (lane & 7) < (warp & 7) ? gs[lane] : 0u);
+    uint32_t incl = all;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    total = all;
+    excl = below + incl - all;
+    uint32_t run = excl + lower;
+#pragma unroll
+    for (int w = 0; w < WPP; ++w) {
+      wcnt_all[(q * WPP + w) * kRadix + d] = run;
+      run += part[w];
+    }
+    __syncthreads();
+
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      if (valid(i)) {
+        const uint32_t p = wc[digit_of(key[i], shift, mask, dxor)] + ((i & 1) ? rank2[i / 2] >> 16 : rank2[i / 2] & 0xFFFFu);
+        kb[p] = key[i];
+        if (PAIRS) vb[p] = val[i];
+      }
+    }
+    __syncwarp();
+    clear_counts(smem);
+    __syncthreads();
+  }
+  // A whole sort of the tile: p passes, then the store.
+  __device__ __forceinline__ void sort(unsigned char* smem, const K* keys_in, const uint32_t* vals_in, K* keys_out,
+                                       uint32_t* vals_out, int places, int begin_bit, int end_bit, uint32_t top_xor,
+                                       uint32_t descending, int flip) {
+    const K* kb = reinterpret_cast<const K*>(smem + kbuf);
+    const uint32_t* vb = reinterpret_cast<const uint32_t*>(smem + vbuf);
+    load_keys(keys_in, flip);
+    if (kValuesFirst) load_values(vals_in);
+    for (int pass = 0; pass < places; ++pass) {
+      const int shift = begin_bit + kRadixBits * pass;
+      const uint32_t mask = (1u << min(kRadixBits, end_bit - shift)) - 1u;
+      if (pass > 0) load_keys(kb);
+      bin(
+          smem, shift, mask, (pass == places - 1 ? top_xor : 0u) ^ (descending ? mask : 0u),
+          [&] {
+            if (pass > 0 || !kValuesFirst) load_values(pass > 0 ? vb : vals_in);
+          },
+          [](uint32_t) {});
+    }
+    for (uint32_t j = threadIdx.x; j < count; j += NT) {
+      const K k = kb[j];
+      keys_out[j] = flip ? flip_from_ordered(k) : k;
+      if (PAIRS) vals_out[j] = vb[j];
+    }
+  }
+};
+
+}  // namespace onesweep
