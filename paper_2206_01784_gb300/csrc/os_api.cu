@@ -126,7 +126,7 @@ uint32_t min_tile_keys(int key_bits, bool pairs) {
 
 cudaError_t launch_binning(int key_bits, bool pairs, int cfg, const PassArgs& a, cudaStream_t s, int radix_bits) {
   const int flip = (a.flip_in ? 1 : 0) | (a.flip_out ? 2 : 0);
-  const int seg = a.seg_offsets != nullptr;
+  const int seg = a.tile_desc != nullptr;
   if (radix_bits != kRadixBits) {
     if (seg || radix_bits < kMinRadixBits || radix_bits > kRadixBits) return cudaErrorInvalidValue;
     return kBinningLaunchRb[key_bits == 64][radix_bits - kMinRadixBits](pairs, flip, a, s);
@@ -569,8 +569,11 @@ constexpr uint64_t kMaxBatchKeys = 1ull << 31;  // total keys of a batch (32-bit
 constexpr uint64_t kMaxSegments = 1ull << 24;
 
 // Batch header words (same header as a single sort): 0 status, 2 binning
-// tiles, 3 histogram items, 4 invalid-offsets flag, 16.. tile counters.
+// tiles, 3 histogram items, 4-6 segments of each one-block class, 8-10 the next
+// of each to be sorted, 16.. tile counters.
 constexpr size_t kTotalsWord = 2;
+constexpr size_t kClassCountWord = 4;
+constexpr size_t kClassNextWord = 8;
 
 struct BatchPlan {
   int key_bits = 0;
@@ -580,10 +583,13 @@ struct BatchPlan {
   int64_t fault_tile = -1;  // test hooks, read once
   uint32_t spin_limit = 0;
   int places = 0;
-  uint32_t tile = 0, small_max = 0;
-  uint64_t max_tiles = 0, max_items = 0;
-  size_t seg_done = 0, seg_skew = 0, seg_hist = 0, zero_end = 0, seg_bin_offsets = 0, tile_base = 0, hist_base = 0;
-  size_t tile_seg = 0, hist_seg = 0, status[2] = {0, 0}, alt_keys = 0, alt_vals = 0, total = 0;
+  uint32_t tile = 0;
+  uint64_t max_large = 0;    // segments beyond the one-block sorts
+  uint64_t max_tiles = 0, max_items = 0;  // capacities (any tile geometry)
+  uint64_t grid_tiles = 0;   // tiles at most, with this plan's tile
+  size_t seg_done = 0, seg_hist = 0, zero_end = 0, seg_skew = 0, seg_bin_offsets = 0, large_range = 0, tile_base = 0;
+  size_t hist_base = 0, class_list = 0, hist_large = 0, tile_desc = 0, status[2] = {0, 0};
+  size_t alt_keys = 0, alt_vals = 0, total = 0;
 };
 
 int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int value_bytes, int begin_bit,
@@ -602,33 +608,54 @@ int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int va
   bp->cfg = cfg_override >= 0 ? cfg_override : binning_config(kb, bp->pairs, bp->bucket);
   bp->fault_tile = g_fault_tile.load(std::memory_order_relaxed);
   bp->spin_limit = g_spin_limit.load(std::memory_order_relaxed);
+  // the default variant takes smaller tiles while the batch is small: with
+  // little more than one wave of blocks a pass takes as long as a tile, and
+  // short segments fill the larger tiles poorly (us a batch with geometry 0 / 1
+  // / 2: 298 segments, 1.8M f32 pairs 125 / 110 / 107; 232, 3.1M f32 pairs 168 /
+  // 148 / 143; 256, 8.8M i32 keys 220 / 232 / 232; 16, 0.1M f64 keys 111 / 103 /
+  // 92; 76, 1.6M f64 pairs 185 / 173 / 194)
+  if (cfg_override < 0 && bp->cfg == kDefaultTileConfig) {
+    const uint64_t wave = kb == 32 ? 4u << 20 : 5u << 18;
+    if (n_total <= wave)
+      bp->cfg += 2;
+    else if (n_total <= (kb == 32 ? wave : 2 * wave))
+      bp->cfg += 1;
+  }
   // the persistent kernel serves single arrays: a batch runs geometry 0 with
   // the same ranking
   if (bp->cfg % kGeometries == kPersistentGeometry) bp->cfg -= kPersistentGeometry;
   bp->tile = tile_keys_for(kb, bp->pairs, bp->cfg);
-  bp->small_max = batch_local_capacity(kb, bp->pairs);
   const uint32_t min_tile = min_tile_keys(kb, bp->pairs);
-  bp->max_tiles = (n_total + min_tile - 1) / min_tile + S;
-  bp->max_items = (n_total + kHistChunk - 1) / kHistChunk + S;
+  // (n_total keys that fit class 1 make no large segment)
+  bp->max_large = n_total > batch_class_capacity(kb, kBatchClasses - 1) ? n_total / (batch_class_capacity(kb, 0) + 1) : 0;
+  if (bp->max_large > S) bp->max_large = S;
+  bp->max_tiles = n_total / min_tile + bp->max_large;
+  bp->grid_tiles = n_total / bp->tile + bp->max_large;
+  bp->max_items = n_total / kHistChunk + bp->max_large;
+  const uint64_t M = bp->max_large;
   const size_t per_seg = (size_t)(bp->places > 0 ? bp->places : 1) * kRadix * 4;
   size_t off = kHeaderBytes;
   bp->seg_done = off;
-  off = round_up(off + S * 4);
-  bp->seg_skew = off;
-  off = round_up(off + S * (size_t)(bp->places > 0 ? bp->places : 1) * 4);
+  off = round_up(off + M * 4);
   bp->seg_hist = off;
-  off = round_up(off + S * per_seg);
+  off = round_up(off + M * per_seg);
   bp->zero_end = off;
+  bp->seg_skew = off;
+  off = round_up(off + M * (size_t)(bp->places > 0 ? bp->places : 1) * 4);
   bp->seg_bin_offsets = off;
-  off = round_up(off + S * per_seg);
+  off = round_up(off + M * per_seg);
+  bp->large_range = off;
+  off = round_up(off + M * sizeof(uint2));
   bp->tile_base = off;
-  off = round_up(off + (S + 1) * 4);
+  off = round_up(off + (M + 1) * 4);
   bp->hist_base = off;
-  off = round_up(off + (S + 1) * 4);
-  bp->tile_seg = off;
-  off = round_up(off + bp->max_tiles * 4);
-  bp->hist_seg = off;
+  off = round_up(off + (M + 1) * 4);
+  bp->class_list = off;
+  off = round_up(off + S * kBatchClasses * 4);
+  bp->hist_large = off;
   off = round_up(off + bp->max_items * 4);
+  bp->tile_desc = off;
+  off = round_up(off + bp->max_tiles * sizeof(uint4));
   const size_t slab = (size_t)bp->max_tiles * kRadix * 4;
   bp->status[0] = off;
   off = round_up(off + slab);
@@ -697,15 +724,20 @@ int run_batch(int key_type, const void* keys_in, void* keys_out, const uint32_t*
   b.num_places = bp.places;
   b.begin_bit = begin_bit;
   b.end_bit = end_bit;
-  b.small_max = bp.small_max;
+  for (int c = 0; c < kBatchClasses; ++c) b.class_max[c] = batch_class_capacity(bp.key_bits, c);
   b.tile_keys = bp.tile;
   b.hist_chunk = kHistChunk;
+  b.max_large = (uint32_t)bp.max_large;
   b.max_tiles = (uint32_t)bp.max_tiles;
   b.max_items = (uint32_t)bp.max_items;
+  b.class_list = reinterpret_cast<uint32_t*>(w + bp.class_list);
+  b.class_count = header + kClassCountWord;
+  b.class_next = header + kClassNextWord;
+  b.large_range = reinterpret_cast<uint2*>(w + bp.large_range);
   b.tile_base = reinterpret_cast<uint32_t*>(w + bp.tile_base);
-  b.tile_seg = reinterpret_cast<uint32_t*>(w + bp.tile_seg);
   b.hist_base = reinterpret_cast<uint32_t*>(w + bp.hist_base);
-  b.hist_seg = reinterpret_cast<uint32_t*>(w + bp.hist_seg);
+  b.hist_large = reinterpret_cast<uint32_t*>(w + bp.hist_large);
+  b.tile_desc = reinterpret_cast<uint4*>(w + bp.tile_desc);
   b.totals = header + kTotalsWord;
   b.seg_done = reinterpret_cast<uint32_t*>(w + bp.seg_done);
   b.seg_hist = reinterpret_cast<uint32_t*>(w + bp.seg_hist);
@@ -715,18 +747,20 @@ int run_batch(int key_type, const void* keys_in, void* keys_out, const uint32_t*
   b.descending = is_descending(key_type) ? 1u : 0u;
   b.error = header;
   b.clear = reinterpret_cast<uint32_t*>(w + bp.status[0]);
-  b.clear_words = bp.max_tiles * kRadix;
 
   int slot = prof_begin(2, -1, s);
   cudaError_t e = launch_batch_plan(b, s);
   prof_end(slot, s);
   if (e != cudaSuccess) return OS_ERR_CUDA;
-  slot = prof_begin(0, -1, s);
-  e = launch_batch_histogram(bp.key_bits, b, s);
+  slot = prof_begin(3, -1, s);
+  bool after_class = false;
+  e = launch_batch_class_sorts(bp.key_bits, pairs, b, &after_class, s);
   prof_end(slot, s);
   if (e != cudaSuccess) return OS_ERR_CUDA;
-  slot = prof_begin(3, -1, s);
-  e = launch_batch_local_sort(bp.key_bits, pairs, b, s);
+  if (bp.max_large == 0) return OS_OK;  // n_total is too small for a large segment
+  slot = prof_begin(0, -1, s);
+  if (slot >= 0) after_class = false;  // (an event between the two: timed apart)
+  e = launch_batch_histogram(bp.key_bits, b, after_class, s);
   prof_end(slot, s);
   if (e != cudaSuccess) return OS_ERR_CUDA;
 
@@ -745,7 +779,7 @@ int run_batch(int key_type, const void* keys_in, void* keys_out, const uint32_t*
     a.vals_in = pairs ? src_v : nullptr;
     a.vals_out = pairs ? dst_v : nullptr;
     a.n = (uint32_t)n_total;
-    a.num_tiles = (uint32_t)bp.max_tiles;
+    a.num_tiles = (uint32_t)bp.grid_tiles;
     a.shift = begin_bit + kRadixBits * pass;
     const int width = end_bit - a.shift < kRadixBits ? end_bit - a.shift : kRadixBits;
     a.mask = (1u << width) - 1u;
@@ -756,14 +790,12 @@ int run_batch(int key_type, const void* keys_in, void* keys_out, const uint32_t*
     a.offsets_stride = (uint32_t)bp.places * kRadix;
     a.status = reinterpret_cast<uint32_t*>(w + bp.status[pass & 1]);
     a.status_clear = pass + 1 < bp.places ? reinterpret_cast<uint32_t*>(w + bp.status[(pass + 1) & 1]) : nullptr;
-    a.status_clear_rows = (uint32_t)bp.max_tiles;  // every tile clears its own row
+    a.status_clear_rows = (uint32_t)bp.grid_tiles;  // every tile clears its own row
     a.tile_counter = header + kTileCounterWord + pass % 8;
     a.error = header;
     a.spin_limit = bp.spin_limit;
     a.fault_tile = bp.fault_tile;
-    a.seg_offsets = seg_offsets;
-    a.tile_base = b.tile_base;
-    a.tile_seg = b.tile_seg;
+    a.tile_desc = b.tile_desc;
     a.total_tiles = b.totals;
     a.skew_flags = b.seg_skew + pass;
     a.skew_stride = (uint32_t)bp.places;

@@ -4,22 +4,26 @@
 // chain. What this file adds around the binning kernel:
 //
 //  * plan: one block reads the segment boundaries on the device and lays out
-//    the work - each large segment's binning tiles get consecutive tile ids
-//    (its look-back chain) and histogram work items; small segments are left
-//    to the one-block sort. Nothing is read back to the host, so a batch can
-//    be captured in a CUDA graph;
-//  * per-segment histograms: work items of up to kHistChunk keys count the
-//    digits of every place into their segment's histograms; the item that
-//    finishes a segment last takes the exclusive sums (the segment's bin
-//    offsets), as the single-array histogram kernel does for the whole array;
-//  * small segments (up to one block's capacity) are sorted entirely in
-//    shared memory: p in-block binning passes, one global read and one write.
-#include "os_binning.cuh"
-#include "os_common.cuh"
-#include "os_internal.h"
+//    the work. Segments of up to one block's capacity are listed by class for
+//    the one-block sorts; each longer ("large") segment gets a row of its own, consecutive tile ids (its look-back chain) and histogram work items.
+//    Nothing is read back to the host, so a batch can be captured in a CUDA
+//    graph;
+//  * one-block sorts: blocks take the listed segments one after another and
+//    sort each on the chip (SmallTile): one global read and one write;
+//  * histograms of the large segments: work items of up to kHistChunk keys
+//    count the digits of every place into their segment's histograms; the item
+//    that finishes a segment last takes the exclusive sums (the segment's bin
+//    offsets), as the single-array histogram kernel does for the whole array.
+//    They also write a descriptor per tile for the binning passes.
+//
+// Grids and workspaces are bounded by what n keys can make: a large segment
+// is longer than class 0's capacity, so there are at most n / (capacity + 1) of
+// them whatever the number of segments.
+#include "os_small.cuh"
 
 namespace onesweep {
 
+int device_sm_count();
 int ws_grid(uint32_t num_tiles);  // min(num_tiles, SMs of the current device)
 
 namespace {
@@ -28,52 +32,115 @@ constexpr int kPlanThreads = 1024;
 constexpr int kSegHistThreads = 1024;
 constexpr int kSegHistVec = 4;  // 16-byte loads in flight per thread per step of the segment histogram
 
-__global__ void __launch_bounds__(kPlanThreads) batch_plan_kernel(BatchArgs b) {
-  __shared__ uint32_t tmp_t[kPlanThreads / 32 + 1];
-  __shared__ uint32_t tmp_h[kPlanThreads / 32 + 1];
-  __shared__ uint32_t s_bad;
-  const int tid = threadIdx.x;
-  if (tid == 0) s_bad = 0;
+// Classes of the one-block sorts: a block's threads, keys a thread, and how many
+// blocks fit an SM (64 registers a thread). The smaller a class's blocks, the
+// more of them share an SM and cover one another's barriers; the last class
+// holds the longest segment one block can (by shared memory).
+struct BatchClass {
+  int threads, keys_per_thread, blocks_per_sm;
+  constexpr uint32_t capacity() const { return (uint32_t)(threads * keys_per_thread); }
+};
+constexpr BatchClass kClass32[kBatchClasses] = {{256, 16, 4}, {512, 16, 2}, {1024, 16, 1}};
+constexpr BatchClass kClass64[kBatchClasses] = {{256, 8, 4}, {512, 8, 2}, {1024, 8, 1}};
+
+// Exclusive prefix sum of a pair of words over the block.
+__device__ __forceinline__ uint2 block_exclusive_sum2(uint2 v, uint2* tmp, uint2* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint2 x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y0 = __shfl_up_sync(0xFFFFFFFFu, x.x, o), y1 = __shfl_up_sync(0xFFFFFFFFu, x.y, o);
+    if (lane >= o) {
+      x.x += y0;
+      x.y += y1;
+    }
+  }
+  if (lane == 31) tmp[warp] = x;
   __syncthreads();
-  uint32_t carry_t = 0, carry_h = 0;
-  for (uint32_t base = 0; base < b.num_segments; base += kPlanThreads) {
-    const uint32_t s = base + tid;
-    uint32_t nt = 0, nh = 0;
-    if (s < b.num_segments) {
-      const uint64_t lo = b.seg_offsets[s], hi = b.seg_offsets[s + 1];
-      if (hi < lo || hi > b.n_total || hi - lo >= (1ull << 30)) {
-        s_bad = 1;
-      } else {
-        const uint32_t len = (uint32_t)(hi - lo);
-        if (len > b.small_max) {
-          nt = (len + b.tile_keys - 1) / b.tile_keys;
-          nh = (len + b.hist_chunk - 1) / b.hist_chunk;
-        }
+  if (warp == 0) {
+    const uint2 w = tmp[lane];
+    uint2 s = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y0 = __shfl_up_sync(0xFFFFFFFFu, s.x, o), y1 = __shfl_up_sync(0xFFFFFFFFu, s.y, o);
+      if (lane >= o) {
+        s.x += y0;
+        s.y += y1;
       }
     }
-    uint32_t tot_t = 0, tot_h = 0;
-    const uint32_t et = block_exclusive_sum<kPlanThreads>(nt, tmp_t, &tot_t);
-    const uint32_t eh = block_exclusive_sum<kPlanThreads>(nh, tmp_h, &tot_h);
+    tmp[lane] = make_uint2(s.x - w.x, s.y - w.y);
+    if (lane == 31) tmp[32] = s;
+  }
+  __syncthreads();
+  *total = tmp[32];
+  return make_uint2(tmp[warp].x + x.x - v.x, tmp[warp].y + x.y - v.y);
+}
+
+__global__ void __launch_bounds__(kPlanThreads) batch_plan_kernel(BatchArgs b) {
+  __shared__ uint2 tmp[2][33];
+  const int tid = threadIdx.x;
+  // invalid segments, and the longest one
+  bool bad = false, longest = false;
+  for (uint32_t s = tid; s < b.num_segments; s += kPlanThreads) {
+    const uint64_t lo = b.seg_offsets[s], hi = b.seg_offsets[s + 1];
+    bad |= hi < lo || hi > b.n_total || hi - lo >= (1ull << 30);
+    longest |= hi - lo > b.class_max[kBatchClasses - 1];
+  }
+  bad = __syncthreads_or(bad);
+  // when there are binning passes to run, the segments above class 0 join them:
+  // they add little to passes whose time is mostly fixed, while the longest of
+  // them takes tens of microseconds in one block
+  const uint32_t small_max = __syncthreads_or(longest) ? b.class_max[0] : b.class_max[kBatchClasses - 1];
+  uint32_t tiles = 0, items = 0, large = 0, listed[kBatchClasses] = {0, 0, 0};
+  for (uint32_t base = 0; base < b.num_segments && !bad; base += kPlanThreads) {
+    const uint32_t s = base + tid;
+    uint32_t nt = 0, nh = 0, start = 0, len = 0;
     if (s < b.num_segments) {
-      const uint32_t tb = carry_t + et, hb = carry_h + eh;
-      b.tile_base[s] = tb;
-      b.hist_base[s] = hb;
-      if ((uint64_t)tb + nt <= b.max_tiles)
-        for (uint32_t t = 0; t < nt; ++t) b.tile_seg[tb + t] = s;
-      if ((uint64_t)hb + nh <= b.max_items)
-        for (uint32_t h = 0; h < nh; ++h) b.hist_seg[hb + h] = s;
+      start = (uint32_t)b.seg_offsets[s];
+      len = (uint32_t)(b.seg_offsets[s + 1] - b.seg_offsets[s]);
+      if (len > small_max) {
+        nt = (len + b.tile_keys - 1) / b.tile_keys;
+        nh = (len + b.hist_chunk - 1) / b.hist_chunk;
+      }
     }
-    carry_t += tot_t;
-    carry_h += tot_h;
+    const int cls = len == 0 || nt ? -1 : len <= b.class_max[0] ? 0 : len <= b.class_max[1] ? 1 : 2;
+    // exclusive sums of tiles, items, and (at most 1024 a step, 16 bits each)
+    // of large segments and of each class
+    uint2 work_total, low_total;
+    const uint2 work = block_exclusive_sum2(make_uint2(nt, nh), tmp[0], &work_total);
+    const uint2 rank = block_exclusive_sum2(
+        make_uint2((nt ? 1u : 0u) | (cls == 0 ? 1u << 16 : 0u), (cls == 1 ? 1u : 0u) | (cls == 2 ? 1u << 16 : 0u)),
+        tmp[1], &low_total);
+    if (nt) {
+      const uint32_t li = large + (rank.x & 0xFFFFu), tb = tiles + work.x, hb = items + work.y;
+      if (li < b.max_large && (uint64_t)hb + nh <= b.max_items) {
+        b.large_range[li] = make_uint2(start, len);
+        b.tile_base[li] = tb;
+        b.hist_base[li] = hb;
+        for (uint32_t h = 0; h < nh; ++h) b.hist_large[hb + h] = li;
+      }
+    }
+    if (cls == 0) b.class_list[listed[0] + (rank.x >> 16)] = s;
+    if (cls == 1) b.class_list[b.num_segments + listed[1] + (rank.y & 0xFFFFu)] = s;
+    if (cls == 2) b.class_list[2 * (size_t)b.num_segments + listed[2] + (rank.y >> 16)] = s;
+    tiles += work_total.x;
+    items += work_total.y;
+    large += low_total.x & 0xFFFFu;
+    listed[0] += low_total.x >> 16;
+    listed[1] += low_total.y & 0xFFFFu;
+    listed[2] += low_total.y >> 16;
     __syncthreads();
   }
   if (tid == 0) {
-    b.tile_base[b.num_segments] = carry_t;
-    b.hist_base[b.num_segments] = carry_h;
-    const bool bad = s_bad || carry_t > b.max_tiles || carry_h > b.max_items;
-    b.totals[0] = bad ? 0u : carry_t;
-    b.totals[1] = bad ? 0u : carry_h;
-    b.totals[2] = bad ? 1u : 0u;
+    bad = bad || tiles > b.max_tiles || items > b.max_items || large > b.max_large;
+    if (!bad) {
+      b.tile_base[large] = tiles;
+      b.hist_base[large] = items;
+    }
+    b.totals[0] = bad ? 0u : tiles;
+    b.totals[1] = bad ? 0u : items;
+#pragma unroll
+    for (int c = 0; c < kBatchClasses; ++c) b.class_count[c] = bad ? 0u : listed[c];
     if (bad) atomicOr(b.error, kErrBadSegments);
   }
 }
@@ -113,10 +180,10 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
     uint4* s4 = reinterpret_cast<uint4*>(sh);
     for (int i = tid; i < P * kRadix * C / 4; i += kSegHistThreads) s4[i] = make_uint4(0, 0, 0, 0);
   }
-  // zero the first pass's status slab on the way (grid-stride, 16-byte stores)
-  if (b.clear) {
+  // zero the first pass's status rows on the way (grid-stride, 16-byte stores)
+  {
     uint4* c = reinterpret_cast<uint4*>(b.clear);
-    const uint64_t nv = b.clear_words / 4;
+    const uint64_t nv = (uint64_t)__ldcg(b.totals) * (kRadix / 4);
     for (uint64_t i = (uint64_t)blockIdx.x * kSegHistThreads + tid; i < nv; i += (uint64_t)gridDim.x * kSegHistThreads)
       c[i] = make_uint4(0, 0, 0, 0);
   }
@@ -142,7 +209,7 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
   // (each lane starts at a different copy, so a warp's reads and the zeroing
   // stores hit distinct banks); the flush that completes the segment's work
   // items takes its exclusive sums
-  auto flush = [&](uint32_t seg, uint32_t nitems) {
+  auto flush = [&](uint32_t seg, uint32_t nitems) {  // seg: row of a large segment
     __syncthreads();
     uint32_t* gh = b.seg_hist + (size_t)seg * p * kRadix;
     for (int e = tid; e < p * kRadix; e += kSegHistThreads) {
@@ -158,13 +225,13 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-      const uint32_t items = b.hist_base[seg + 1] - b.hist_base[seg];
+      const uint32_t items = __ldcg(b.hist_base + seg + 1) - __ldcg(b.hist_base + seg);
       s_last = (atomicAdd(b.seg_done + seg, nitems) + nitems == items) ? 1u : 0u;
     }
     __syncthreads();
     if (s_last) {
       __threadfence();
-      const uint32_t len = (uint32_t)(b.seg_offsets[seg + 1] - b.seg_offsets[seg]);
+      const uint32_t len = __ldcg(b.large_range + seg).y;
       uint32_t* go = b.seg_bin_offsets + (size_t)seg * p * kRadix;
       for (int pl = 0; pl < p; ++pl) {
         // descending: bins of the complemented digits (count of t = count of t ^ mask)
@@ -181,22 +248,27 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
   };
 
   // this block's contiguous range of work items
-  const uint32_t total_items = b.totals[1];
+  // (the plan's words are read from L2, as in the class sorts)
+  const uint32_t total_items = __ldcg(b.totals + 1);
   const uint32_t per_block = (total_items + gridDim.x - 1) / gridDim.x;
   const uint32_t it0 = min(blockIdx.x * per_block, total_items);
   const uint32_t it1 = min(it0 + per_block, total_items);
   uint32_t cur = 0xFFFFFFFFu, run = 0;
   for (uint32_t item = it0; item < it1; ++item) {
-    const uint32_t seg = b.hist_seg[item];
+    const uint32_t seg = __ldcg(b.hist_large + item);
     if (seg != cur) {
       if (run) flush(cur, run);
       cur = seg;
       run = 0;
     }
-    const uint64_t s0 = b.seg_offsets[seg];
-    const uint32_t len = (uint32_t)(b.seg_offsets[seg + 1] - s0);
-    const uint32_t lo = (item - b.hist_base[seg]) * b.hist_chunk;
+    const uint2 range = __ldcg(b.large_range + seg);
+    const uint32_t s0 = range.x, len = range.y;
+    const uint32_t lo = (item - __ldcg(b.hist_base + seg)) * b.hist_chunk;
     const uint32_t cnt = min(b.hist_chunk, len - lo);
+    // descriptors of the tiles that start in this chunk
+    const uint32_t chain = __ldcg(b.tile_base + seg);
+    for (uint32_t t = (lo + b.tile_keys - 1) / b.tile_keys + tid; t * b.tile_keys < lo + cnt; t += kSegHistThreads)
+      b.tile_desc[chain + t] = make_uint4(s0 + t * b.tile_keys, len, chain, seg);
     const K* keys = static_cast<const K*>(b.keys_in) + s0 + lo;
     // 16-byte vectors between an unaligned head and a tail of fewer than PER_VEC keys
     const uintptr_t addr = reinterpret_cast<uintptr_t>(keys);
@@ -226,141 +298,84 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
     ++run;
   }
   if (run) flush(cur, run);
+  if (blockIdx.x == 0) pdl_wait();  // the class sorts before this kernel have ended when it ends
 }
 
-// One-block sort of a small segment (up to LocalConfig::T keys).
-template <int KBITS>
-struct LocalConfig {
-  static constexpr int NT = 256;
-  static constexpr int IPT = KBITS == 32 ? 16 : 8;
-  static constexpr int T = NT * IPT;
-  static constexpr int NW = NT / 32;
+// One-block sorts of one class's segments: resident blocks take them one after
+// another. The classes and the histogram kernel after them work on different
+// segments, so each is launched to start when the one before has started
+// (programmatic dependent launch) and fills the SMs that it leaves idle. Block 0
+// waits for the kernel before to complete before it ends itself: what the
+// stream runs after the last of them then follows them all.
+template <int KBITS, bool PAIRS, int CLS>
+struct ClassTile {
+  static constexpr BatchClass kClass = KBITS == 32 ? kClass32[CLS] : kClass64[CLS];
+  using Tile = SmallTile<KBITS, PAIRS, kClass.threads, kClass.keys_per_thread, true, true>;
+  static_assert(kClass.blocks_per_sm * (Tile::smem_bytes + 1024) <= 228 * 1024, "blocks of a class on an SM");
 };
 
-template <int KBITS, bool PAIRS>
-constexpr size_t local_smem_bytes() {
-  using L = LocalConfig<KBITS>;
-  return (size_t)L::T * (KBITS / 8) + (PAIRS ? (size_t)L::T * 4 : 0) + (size_t)L::NW * kRadix * 4 + 64 * 4;
-}
-
-template <int KBITS, bool PAIRS>
-__global__ void __launch_bounds__(LocalConfig<KBITS>::NT) batch_local_sort_kernel(BatchArgs b) {
-  using L = LocalConfig<KBITS>;
-  using K = typename KeyWord<KBITS>::type;
-  constexpr int NT = L::NT, IPT = L::IPT, NW = L::NW, U = rank_chunk(PAIRS, IPT);
+template <int KBITS, bool PAIRS, int CLS>
+__global__ void __launch_bounds__(ClassTile<KBITS, PAIRS, CLS>::kClass.threads, ClassTile<KBITS, PAIRS, CLS>::kClass.blocks_per_sm)
+    batch_class_sort_kernel(BatchArgs b) {
+  using Tile = typename ClassTile<KBITS, PAIRS, CLS>::Tile;
+  using K = typename Tile::K;
   extern __shared__ __align__(128) unsigned char smem[];
-  K* kbuf = reinterpret_cast<K*>(smem);
-  uint32_t* vbuf = reinterpret_cast<uint32_t*>(smem + (size_t)L::T * sizeof(K));
-  uint32_t* whist = reinterpret_cast<uint32_t*>(smem + (size_t)L::T * sizeof(K) + (PAIRS ? (size_t)L::T * 4 : 0));
-  uint32_t* misc = whist + NW * kRadix;
-
-  const uint32_t seg = blockIdx.x;
-  if (seg >= b.num_segments || b.totals[2]) return;
-  const uint64_t s0 = b.seg_offsets[seg];
-  const uint32_t len = (uint32_t)(b.seg_offsets[seg + 1] - s0);
-  if (len == 0 || len > b.small_max || len > (uint32_t)L::T) return;
-
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const K* kin = static_cast<const K*>(b.keys_in) + s0;
-  for (uint32_t i = tid; i < len; i += NT) kbuf[i] = b.flip ? flip_to_ordered(kin[i]) : kin[i];
-  if (PAIRS)
-    for (uint32_t i = tid; i < len; i += NT) vbuf[i] = b.vals_in[s0 + i];
-
-  uint32_t* wcnt = whist;  // [NW][256] digit counts
-  uint32_t* wc = wcnt + warp * kRadix;
-  const uint32_t wbase = (uint32_t)warp * IPT * 32 + lane;
-  for (int pass = 0; pass < b.num_places; ++pass) {
-    const int shift = b.begin_bit + 8 * pass;
-    const int width = min(8, b.end_bit - shift);
-    const uint32_t mask = (1u << width) - 1u;
-    const uint32_t dxor = (pass == b.num_places - 1 ? b.top_xor : 0u) ^ (b.descending ? mask : 0u);
-    for (int i = tid; i < NW * kRadix; i += NT) whist[i] = 0;
-    __syncthreads();  // staged keys (or the previous pass's scatter) visible
-    K key[IPT];
-    const K first = kbuf[0];
-    const K digit_bits = (K)mask << shift;
-    K differ = 0;
-#pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      const uint32_t idx = wbase + i * 32;
-      key[i] = idx < len ? kbuf[idx] : K(0);
-      if (idx < len) differ |= (key[i] ^ first) & digit_bits;
-    }
-    if (__syncthreads_or(differ != 0) == 0) continue;  // one digit: order unchanged
-
-    uint32_t rank[IPT];
-#pragma unroll
-    for (int i0 = 0; i0 < IPT; i0 += U) {
-      uint32_t d[U], r[U];
-      bool valid[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        valid[u] = wbase + (i0 + u) * 32 < len;
-        d[u] = digit_of(key[i0 + u], shift, mask, dxor);
-      }
-      rank_atomic<false, U>(wc, d, valid, r);
-#pragma unroll
-      for (int u = 0; u < U; ++u) rank[i0 + u] = r[u];
-    }
+  __shared__ uint32_t s_item;
+  pdl_launch_dependents();
+  // (what the plan wrote is read from L2: this kernel may start while the one
+  // before it, which the plan's completion let start, is still running)
+  const uint32_t items = __ldcg(b.class_count + CLS);
+  const uint32_t* list = b.class_list + (size_t)CLS * b.num_segments;
+  for (;;) {
+    if (threadIdx.x == 0) s_item = atomicAdd(b.class_next + CLS, 1u);
     __syncthreads();
-    uint32_t total = 0;
-    if (tid < kRadix)
-      for (int w = 0; w < NW; ++w) total += wcnt[w * kRadix + tid] & 0xFFFFu;  // (the high halves hold lane sums)
-    const uint32_t excl = block_exclusive_sum<NT>(tid < kRadix ? total : 0u, misc);
-    if (tid < kRadix) {
-      uint32_t run = excl;
-      for (int w = 0; w < NW; ++w) {
-        const uint32_t cw = wcnt[w * kRadix + tid] & 0xFFFFu;
-        wcnt[w * kRadix + tid] = run;
-        run += cw;
-      }
-    }
-    __syncthreads();
-    uint32_t pos[IPT];
-    uint32_t val[PAIRS ? IPT : 1];
-#pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      const uint32_t idx = wbase + i * 32;
-      const bool valid = idx < len;
-      pos[i] = valid ? wc[digit_of(key[i], shift, mask, dxor)] + rank[i] : 0u;
-      if (PAIRS) val[i] = valid ? vbuf[idx] : 0u;
-    }
-    __syncthreads();  // every read of the old order is done
-#pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      if (wbase + i * 32 < len) {
-        kbuf[pos[i]] = key[i];
-        if (PAIRS) vbuf[pos[i]] = val[i];
-      }
-    }
+    const uint32_t item = s_item;
+    if (item >= items) break;
+    const uint32_t seg = __ldcg(list + item);
+    const uint64_t s0 = b.seg_offsets[seg];
+    Tile t;
+    t.init(smem, (uint32_t)(b.seg_offsets[seg + 1] - s0));
+    t.sort(smem, static_cast<const K*>(b.keys_in) + s0, PAIRS ? b.vals_in + s0 : nullptr,
+           static_cast<K*>(b.keys_out) + s0, PAIRS ? b.vals_out + s0 : nullptr, b.num_places, b.begin_bit, b.end_bit,
+           b.top_xor, b.descending, b.flip);
+    __syncthreads();  // everyone has read s_item and the sorted tile
   }
-  __syncthreads();
-  K* kout = static_cast<K*>(b.keys_out) + s0;
-  for (uint32_t i = tid; i < len; i += NT) kout[i] = b.flip ? flip_from_ordered(kbuf[i]) : kbuf[i];
-  if (PAIRS)
-    for (uint32_t i = tid; i < len; i += NT) b.vals_out[s0 + i] = vbuf[i];
+  if (blockIdx.x == 0) pdl_wait();
 }
 
+template <int KBITS, bool PAIRS, int CLS>
+cudaError_t launch_class(const BatchArgs& b, bool* after_kernel, cudaStream_t s) {
+  using CT = ClassTile<KBITS, PAIRS, CLS>;
+  auto* kernel = batch_class_sort_kernel<KBITS, PAIRS, CLS>;
+  // set on every launch: an idempotent host-side attribute
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CT::Tile::smem_bytes);
+  if (e != cudaSuccess) return e;
+  const int sms = device_sm_count();
+  if (sms <= 0) return cudaErrorInvalidConfiguration;
+  // at most one block per segment the class can have, by the class below's capacity
+  uint64_t grid = CLS == 0 ? b.n_total : b.n_total / (b.class_max[CLS == 0 ? 0 : CLS - 1] + 1);
+  if (grid > b.num_segments) grid = b.num_segments;
+  if (grid > (uint64_t)sms * CT::kClass.blocks_per_sm) grid = (uint64_t)sms * CT::kClass.blocks_per_sm;
+  if (grid == 0) return cudaSuccess;
+  e = launch_kernel(kernel, (unsigned)grid, CT::kClass.threads, CT::Tile::smem_bytes, s, *after_kernel, b);
+  *after_kernel = true;
+  return e;
+}
+
+// the longest first, so that the shorter sorts fill the gaps at the end. The
+// first of them waits for the plan as any kernel does.
 template <int KBITS, bool PAIRS>
-cudaError_t launch_local(const BatchArgs& b, cudaStream_t s) {
-  constexpr size_t bytes = local_smem_bytes<KBITS, PAIRS>();
-  static int configured_device = -1;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (configured_device != dev) {
-    cudaError_t e =
-        cudaFuncSetAttribute(batch_local_sort_kernel<KBITS, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return e;
-    configured_device = dev;
-  }
-  batch_local_sort_kernel<KBITS, PAIRS><<<b.num_segments, LocalConfig<KBITS>::NT, bytes, s>>>(b);
-  return cudaGetLastError();
+cudaError_t launch_classes(const BatchArgs& b, bool* after_class, cudaStream_t s) {
+  cudaError_t e = launch_class<KBITS, PAIRS, 2>(b, after_class, s);
+  if (e == cudaSuccess) e = launch_class<KBITS, PAIRS, 1>(b, after_class, s);
+  if (e == cudaSuccess) e = launch_class<KBITS, PAIRS, 0>(b, after_class, s);
+  return e;
 }
 
 }  // namespace
 
-uint32_t batch_local_capacity(int key_bits, bool) {
-  return key_bits == 32 ? LocalConfig<32>::T : LocalConfig<64>::T;
+uint32_t batch_class_capacity(int key_bits, int cls) {
+  return key_bits == 32 ? kClass32[cls].capacity() : kClass64[cls].capacity();
 }
 
 cudaError_t launch_batch_plan(const BatchArgs& b, cudaStream_t s) {
@@ -369,26 +384,28 @@ cudaError_t launch_batch_plan(const BatchArgs& b, cudaStream_t s) {
 }
 
 template <int KBITS>
-cudaError_t launch_batch_histogram_t(const BatchArgs& b, int grid, cudaStream_t s) {
+cudaError_t launch_batch_histogram_t(const BatchArgs& b, int grid, bool after_class, cudaStream_t s) {
   constexpr size_t bytes = BatchHistLayout<KBITS>::smem_bytes;
   // set on every launch: an idempotent host-side attribute
   cudaError_t e = cudaFuncSetAttribute(batch_histogram_kernel<KBITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)bytes);
   if (e != cudaSuccess) return e;
-  batch_histogram_kernel<KBITS><<<grid, kSegHistThreads, bytes, s>>>(b);
-  return cudaGetLastError();
+  return launch_kernel(batch_histogram_kernel<KBITS>, (unsigned)grid, kSegHistThreads, bytes, s, after_class, b);
 }
 
-cudaError_t launch_batch_histogram(int key_bits, const BatchArgs& b, cudaStream_t s) {
+cudaError_t launch_batch_histogram(int key_bits, const BatchArgs& b, bool after_class, cudaStream_t s) {
   // one block per SM (128 KiB of shared memory each), at most one per work item
   const int grid = ws_grid(b.max_items > 0 ? b.max_items : 1u);
   if (grid <= 0) return cudaErrorInvalidConfiguration;
-  return key_bits == 32 ? launch_batch_histogram_t<32>(b, grid, s) : launch_batch_histogram_t<64>(b, grid, s);
+  return key_bits == 32 ? launch_batch_histogram_t<32>(b, grid, after_class, s)
+                        : launch_batch_histogram_t<64>(b, grid, after_class, s);
 }
 
-cudaError_t launch_batch_local_sort(int key_bits, bool pairs, const BatchArgs& b, cudaStream_t s) {
-  if (key_bits == 32) return pairs ? launch_local<32, true>(b, s) : launch_local<32, false>(b, s);
-  return pairs ? launch_local<64, true>(b, s) : launch_local<64, false>(b, s);
+cudaError_t launch_batch_class_sorts(int key_bits, bool pairs, const BatchArgs& b, bool* after_class, cudaStream_t s) {
+  *after_class = false;
+  if (key_bits == 32)
+    return pairs ? launch_classes<32, true>(b, after_class, s) : launch_classes<32, false>(b, after_class, s);
+  return pairs ? launch_classes<64, true>(b, after_class, s) : launch_classes<64, false>(b, after_class, s);
 }
 
 }  // namespace onesweep

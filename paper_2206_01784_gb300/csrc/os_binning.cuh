@@ -575,19 +575,18 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
     TileCtx c{};
     c.tile = tile;
     if (SEG) {
-      if (tile < *a.total_tiles) {
-        const uint32_t seg = a.tile_seg[tile];
-        const uint64_t s0 = a.seg_offsets[seg];
-        const uint32_t len = (uint32_t)(a.seg_offsets[seg + 1] - s0);
-        c.chain_first = a.tile_base[seg];
-        const uint32_t local = (tile - c.chain_first) * (uint32_t)T;
-        if (local < len) {
-          c.start = (uint32_t)s0 + local;
-          c.count = min((uint32_t)T, len - local);
-          c.out_base = (uint32_t)s0;
-          c.out_len = len;
-          c.bin_offsets = a.bin_offsets + (size_t)seg * a.offsets_stride;
-          if (RANK == kRankAdaptive && a.skew_flags) c.skewed = a.skew_flags[(size_t)seg * a.skew_stride];
+      // (the descriptor and the number of tiles are read together)
+      const uint4 d = tile < a.num_tiles ? a.tile_desc[tile] : make_uint4(0, 0, 0, 0);
+      if (tile < min(*a.total_tiles, a.num_tiles)) {
+        c.chain_first = d.z;
+        const uint32_t local = (tile - d.z) * (uint32_t)T;
+        if (local < d.y) {
+          c.start = d.x;
+          c.count = min((uint32_t)T, d.y - local);
+          c.out_base = d.x - local;
+          c.out_len = d.y;
+          c.bin_offsets = a.bin_offsets + (size_t)d.w * a.offsets_stride;
+          if (RANK == kRankAdaptive && a.skew_flags) c.skewed = a.skew_flags[(size_t)d.w * a.skew_stride];
         }
       }
     } else if (tile < a.num_tiles) {
@@ -624,9 +623,18 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
     }
     // the tile kPrefetchTiles ahead starts well within one block lifetime:
     // bring it into L2 now, so its staging copy reads L2 instead of DRAM
-    if (!SEG && a.use_bulk && tile + kPrefetchTiles < a.num_tiles &&
-        (uint64_t)(tile + kPrefetchTiles + 1) * T <= a.n) {
-      const size_t first = (size_t)(tile + kPrefetchTiles) * T;
+    const uint32_t ahead = tile + kPrefetchTiles;
+    if (SEG && a.use_bulk && c.count > 0 && ahead < min(*a.total_tiles, a.num_tiles)) {
+      // whole 16-byte words from the one holding the tile's first key
+      const uint4 d = a.tile_desc[ahead];
+      const uint32_t end = d.x + min((uint32_t)T, d.y - (ahead - d.z) * (uint32_t)T);
+      const uint32_t ks = d.x & ~(kKeysPer16B - 1u), vs = d.x & ~3u;
+      const uint32_t kbytes = ((end - ks) * (uint32_t)sizeof(K)) & ~15u, vbytes = ((end - vs) * 4u) & ~15u;
+      if (kbytes) bulk_prefetch_l2(static_cast<const K*>(a.keys_in) + ks, kbytes);
+      if (PAIRS && vbytes) bulk_prefetch_l2(a.vals_in + vs, vbytes);
+    }
+    if (!SEG && a.use_bulk && ahead < a.num_tiles && (uint64_t)(ahead + 1) * T <= a.n) {
+      const size_t first = (size_t)ahead * T;
       bulk_prefetch_l2(static_cast<const K*>(a.keys_in) + first, (uint32_t)(T * sizeof(K)));
       if (PAIRS) bulk_prefetch_l2(a.vals_in + first, (uint32_t)T * 4u);
     }

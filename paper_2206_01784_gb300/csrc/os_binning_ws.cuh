@@ -648,7 +648,7 @@ cudaError_t launch_binning_flip_rank(const PassArgs& a, cudaStream_t s, int cfg)
     case 3:
       // the persistent kernel serves one array (strips included); a batch
       // keeps geometry 0 (its plan is made with that tile)
-      if (!SEG) return launch_binning_ws<KBITS, PAIRS, RANK, FLIP>(a, s);
+      if constexpr (!SEG) return launch_binning_ws<KBITS, PAIRS, RANK, FLIP>(a, s);
       return launch_binning_one<KBITS, PAIRS, 0, RANK, FLIP, SEG>(a, s);
     default: return launch_binning_one<KBITS, PAIRS, 0, RANK, FLIP, SEG>(a, s);
   }

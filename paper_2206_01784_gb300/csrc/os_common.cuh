@@ -146,6 +146,13 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
+// Programmatic dependent launch: lets the stream's next kernel (when launched
+// with that attribute) start once every block of this one has said so or has
+// ended; and waits until the kernel before this one has completed and its
+// memory operations are visible (no-ops in kernels launched without it).
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- block scan
 
 // Exclusive prefix sum over the NT threads of a block (each contributes v).

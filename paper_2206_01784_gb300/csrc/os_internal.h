@@ -8,6 +8,24 @@
 
 namespace onesweep {
 
+// Launches a one-argument kernel; early: it may start once every block of the
+// stream's last kernel has called pdl_launch_dependents or has ended.
+template <typename Args>
+cudaError_t launch_kernel(void (*kernel)(Args), unsigned grid, unsigned threads, size_t smem_bytes, cudaStream_t s,
+                          bool early, const Args& args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem_bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
 // Phase 1 + 2 (Section 3, "Upfront histogram kernel", "Exclusive sum kernel").
 struct HistArgs {
   const void* keys;          // n keys (device)
@@ -58,12 +76,12 @@ struct PassArgs {
   uint32_t out_total;
   uint32_t* carry_out;
 
-  // Segmented mode (os_sort_batch); seg_offsets == nullptr means one array of
-  // n keys. Each segment is its own sort: its tiles form one look-back chain
-  // and it has its own bin offsets.
-  const uint64_t* seg_offsets;   // [S+1] segment boundaries (device)
-  const uint32_t* tile_base;     // [S+1] first tile of each segment's chain
-  const uint32_t* tile_seg;      // [tiles] segment of each tile
+  // Segmented mode (os_sort_batch); tile_desc == nullptr means one array of n
+  // keys. Each large segment is its own sort: its tiles form one look-back
+  // chain and it has its own bin offsets. A tile's descriptor: array index of
+  // its first key, its segment's length, its chain's first tile, its segment's
+  // row (bin offsets, skew flags).
+  const uint4* tile_desc;        // [tiles]
   const uint32_t* total_tiles;   // device word: tiles in this pass
   uint32_t offsets_stride;       // words between two segments' bin offsets
 
@@ -102,8 +120,9 @@ uint32_t small_blocks(int form, uint64_t n);
 bool small_needs_matrices(int form);  // exchanges counts through SmallArgs::counts_*
 cudaError_t launch_small(int key_bits, bool pairs, int form, const SmallArgs& a, cudaStream_t s);
 
-// Segmented sort: the plan, per-segment histograms and the one-block sort of
-// small segments (os_batch.cu).
+// Segmented sort: the plan, the histograms of the large segments and the
+// one-block sorts of the others (os_batch.cu).
+constexpr int kBatchClasses = 3;  // of the one-block sorts
 struct BatchArgs {
   const void* keys_in;
   void* keys_out;
@@ -116,33 +135,39 @@ struct BatchArgs {
   int num_places;
   int begin_bit;
   int end_bit;
-  uint32_t small_max;            // segments up to this length are sorted in one block
+  uint32_t class_max[kBatchClasses];  // longest segment of each class of the one-block sorts
   uint32_t tile_keys;            // binning tile of the large segments
   uint32_t hist_chunk;           // keys per histogram work item
-  uint32_t max_tiles;            // capacity of tile_seg
-  uint32_t max_items;            // capacity of hist_seg
-  uint32_t* tile_base;           // [S+1]
-  uint32_t* tile_seg;            // [max_tiles]
-  uint32_t* hist_base;           // [S+1]
-  uint32_t* hist_seg;            // [max_items]
+  uint32_t max_large;            // capacity of the large segments' rows
+  uint32_t max_tiles;            // capacity of tile_desc
+  uint32_t max_items;            // capacity of hist_large
+  uint32_t* class_list;          // [kBatchClasses][S] segments of each class
+  uint32_t* class_count;         // [kBatchClasses]
+  uint32_t* class_next;          // [kBatchClasses] zeroed
+  uint2* large_range;            // [max_large] first key, length
+  uint32_t* tile_base;           // [max_large+1] first tile
+  uint32_t* hist_base;           // [max_large+1] first histogram work item
+  uint32_t* hist_large;          // [max_items] row of each work item's segment
+  uint4* tile_desc;              // [max_tiles] (PassArgs::tile_desc)
   uint32_t* totals;              // [0] binning tiles, [1] histogram items
-  uint32_t* seg_done;            // [S] zeroed
-  uint32_t* seg_hist;            // [S][p][256] zeroed
-  uint32_t* seg_bin_offsets;     // [S][p][256]
-  uint32_t* seg_skew;            // [S][p] skewed-place flags
+  uint32_t* seg_done;            // [max_large] zeroed
+  uint32_t* seg_hist;            // [max_large][p][256] zeroed
+  uint32_t* seg_bin_offsets;     // [max_large][p][256]
+  uint32_t* seg_skew;            // [max_large][p] skewed-place flags
   uint32_t top_xor;              // signed keys: high bit of the top place's digit inverted (else 0)
   uint32_t descending;           // bin by the complemented digit of every place
   uint32_t* error;
-  uint32_t* clear;               // status slab of the first pass, to zero
-  uint64_t clear_words;
+  uint32_t* clear;               // status slab of the first pass, whose rows in use are zeroed
 };
 
 constexpr uint32_t kErrBadSegments = 2u;  // device status word bit: invalid segment offsets
 
 cudaError_t launch_batch_plan(const BatchArgs& b, cudaStream_t s);
-cudaError_t launch_batch_histogram(int key_bits, const BatchArgs& b, cudaStream_t s);
-cudaError_t launch_batch_local_sort(int key_bits, bool pairs, const BatchArgs& b, cudaStream_t s);
-uint32_t batch_local_capacity(int key_bits, bool pairs);
+// *after_class: whether the stream's last kernel is now a class sort (which the
+// histogram kernel may overlap).
+cudaError_t launch_batch_class_sorts(int key_bits, bool pairs, const BatchArgs& b, bool* after_class, cudaStream_t s);
+cudaError_t launch_batch_histogram(int key_bits, const BatchArgs& b, bool after_class, cudaStream_t s);
+uint32_t batch_class_capacity(int key_bits, int cls);
 
 // Active binning variant for a key width / payload / size bucket, and the
 // tile size of a variant.

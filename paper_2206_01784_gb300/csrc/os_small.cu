@@ -47,7 +47,8 @@ constexpr int kMaxCluster = 16;
 
 template <int KBITS, bool PAIRS, int NT, int IPT, int SCOPE>
 struct SmallLayout {
-  using Tile = SmallTile<KBITS, PAIRS, NT, IPT>;
+  using Tile = SmallTile<KBITS, PAIRS, NT, IPT, SCOPE == kScopeBlock>;
+  static_assert(Tile::T < (1 << 14), "exchanged counts are 14 bits wide");
   static constexpr bool kCluster = SCOPE == kScopeCluster;
   static constexpr size_t scan = Tile::smem_bytes;                        // [8] scan scratch
   static constexpr size_t gtot = scan + 32;                               // [256] digit totals of all blocks

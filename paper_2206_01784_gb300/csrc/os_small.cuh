@@ -7,9 +7,14 @@
 
 namespace onesweep {
 
-template <int KBITS, bool PAIRS, int NT_, int IPT_>
+// SPREAD: the tile's keys are spread evenly over the block's threads (ceil(n /
+// NT) each) rather than filling the first warps with IPT a thread, so that a
+// tile takes time by its length; for tiles that are whole sorts. APART: a digit
+// that many keys of a warp share is ranked apart.
+template <int KBITS, bool PAIRS, int NT_, int IPT_, bool SPREAD = false, bool APART = false>
 struct SmallTile {
   using K = typename KeyWord<KBITS>::type;
+  static constexpr uint32_t kDominantLanes = 6;  // lanes of the first batch that make a digit dominant
   static constexpr int NT = NT_, IPT = IPT_, NW = NT / 32;
   static constexpr int T = NT * IPT;        // keys per tile
   static constexpr int Q = NT / kRadix;     // parts of 8 warps, whose counts of a digit one thread adds up
@@ -17,7 +22,7 @@ struct SmallTile {
   // with few keys a thread, the first pass's values are loaded beside its keys:
   // both come from DRAM, and there are registers for both
   static constexpr bool kValuesFirst = IPT <= 4;
-  static_assert(NT % kRadix == 0 && Q <= 4 && T < (1 << 14), "tile shape (exchanged counts are 14 bits wide)");
+  static_assert(NT % kRadix == 0 && Q <= 4 && T < (1 << 16), "tile shape (the counters' halves are 16 bits wide)");
   // shared memory (bytes)
   static constexpr size_t kbuf = 0;                                   // the tile in digit order
   static constexpr size_t vbuf = kbuf + (size_t)T * sizeof(K);
@@ -30,18 +35,23 @@ struct SmallTile {
   uint32_t val[PAIRS ? IPT : 1];
   uint32_t count;   // keys in the tile
   uint32_t wbase;   // tile position of this thread's first key
+  int ipt;          // keys of a thread (SPREAD)
   uint32_t total;   // threads 0..255, after bin(): the tile's count of digit tid ...
   uint32_t excl;    // ... and of the digits below it
 
   // This thread's keys: warp-striped, batch i of warp w covers positions
-  // [w*IPT*32 + i*32, +32), so batch order and lane order are tile order.
+  // [w*keys()*32 + i*32, +32), so batch order and lane order are tile order.
   __device__ __forceinline__ void init(unsigned char* smem, uint32_t n) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     count = n;
-    wbase = (uint32_t)warp * IPT * 32 + lane;
+    ipt = SPREAD ? (int)((n + NT - 1) / NT) : IPT;
+    wbase = (uint32_t)warp * keys() * 32 + lane;
     clear_counts(smem);
   }
-  __device__ __forceinline__ bool valid(int i) const { return wbase + i * 32 < count; }
+  __device__ __forceinline__ int keys() const { return SPREAD ? ipt : IPT; }
+  __device__ __forceinline__ bool valid(int i) const {
+    return (!SPREAD || i < ipt) && wbase + i * 32 < count;
+  }
   __device__ __forceinline__ void clear_counts(unsigned char* smem) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint4* row = reinterpret_cast<uint4*>(smem + wcnt) + warp * (kRadix / 4);
@@ -60,9 +70,11 @@ struct SmallTile {
   }
   template <bool kL2 = false>
   __device__ __forceinline__ void load_values(const uint32_t* vals) {
-    if (!PAIRS) return;
+    if constexpr (PAIRS) {
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) val[i] = !valid(i) ? 0u : kL2 ? __ldcg(vals + wbase + i * 32) : vals[wbase + i * 32];
+      for (int i = 0; i < IPT; ++i)
+        val[i] = !valid(i) ? 0u : kL2 ? __ldcg(vals + wbase + i * 32) : vals[wbase + i * 32];
+    }
   }
 
   // One binning pass: on return kbuf (and vbuf) hold the tile in stable digit
@@ -87,32 +99,58 @@ struct SmallTile {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t* wc = wcnt_all + warp * kRadix;
 
-    // rank each key among its warp's equal digits; a warp whose keys share one
-    // digit has nothing to rank (and its atomics would all meet in one counter)
+    // rank each key among its warp's equal digits. A warp whose keys share one
+    // digit has nothing to rank. APART: a digit that many of the warp's first
+    // keys share (the most frequent of four sampled lanes') is ranked by votes,
+    // for its atomics would all meet in one counter
     uint32_t rank2[IPT / 2];  // two 16-bit ranks to a register
     const uint32_t d0 = __shfl_sync(0xFFFFFFFFu, digit_of(key[0], shift, mask, dxor), 0);
     bool differ = false;
 #pragma unroll
     for (int i = 0; i < IPT; ++i) differ |= valid(i) && digit_of(key[i], shift, mask, dxor) != d0;
     if (__any_sync(0xFFFFFFFFu, differ)) {
+      uint32_t dominant = kRadix, most = kDominantLanes - 1, position = 0;
+      if constexpr (APART) {
+        const uint32_t mine = valid(0) ? digit_of(key[0], shift, mask, dxor) : kRadix;
+#pragma unroll
+        for (int l = 0; l < 32; l += 8) {
+          const uint32_t dl = __shfl_sync(0xFFFFFFFFu, mine, l);
+          const uint32_t lanes = __popc(__ballot_sync(0xFFFFFFFFu, mine == dl));
+          if (dl < kRadix && lanes > most) {
+            most = lanes;
+            dominant = dl;
+          }
+        }
+      }
 #pragma unroll
       for (int i0 = 0; i0 < IPT; i0 += U) {
+        if (SPREAD && i0 >= ipt) break;
         uint32_t d[U], r[U];
         bool v[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          v[u] = valid(i0 + u);
           d[u] = digit_of(key[i0 + u], shift, mask, dxor);
+          v[u] = valid(i0 + u) && (!APART || d[u] != dominant);
         }
         rank_atomic<false, U>(wc, d, v, r);
+        if (APART && dominant < kRadix) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const bool same = valid(i0 + u) && d[u] == dominant;
+            const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, same);
+            if (same) r[u] = position + __popc(lanes & lanemask_lt());
+            position += __popc(lanes);
+          }
+        }
 #pragma unroll
         for (int u = 0; u < U; u += 2) rank2[(i0 + u) / 2] = r[u] | r[u + 1] << 16;
       }
+      if (APART && dominant < kRadix && lane == 0) wc[dominant] = position;
     } else {
 #pragma unroll
       for (int i = 0; i < IPT; i += 2) rank2[i / 2] = (i * 32 + lane) | ((i + 1) * 32 + lane) << 16;
-      const uint32_t first = (uint32_t)warp * IPT * 32;
-      if (lane == 0 && count > first) wc[d0] = min((uint32_t)IPT * 32, count - first);
+      const uint32_t first = (uint32_t)warp * keys() * 32;
+      if (lane == 0 && count > first) wc[d0] = min((uint32_t)keys() * 32, count - first);
     }
     values();
     __syncthreads();
