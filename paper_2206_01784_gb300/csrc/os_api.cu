@@ -67,8 +67,8 @@ constexpr int kMaxPlaces = 16;  // 64-bit keys in 5-bit digits: 13 places
 
 // Binning kernel variants: tile geometry (4) x digit-ranking method (3);
 // variant v uses geometry v % 4 and ranking v / 4 (0: one ballot per digit
-// bit; 1: adaptive - ballots where the place is skewed, else counting atomics;
-// 2: counting atomics only).
+// bit; 1: adaptive - counting atomics, one digit apart or ballots by the place's
+// histogram; 2: counting atomics only).
 // Geometries 0-2 run one block per tile; geometry 3 is the persistent,
 // warp-specialised kernel (os_binning_ws.cuh), for single arrays only.
 constexpr int kGeometries = 4;
@@ -153,7 +153,7 @@ constexpr uint32_t kDefaultSpinLimit = 1u << 22;
 constexpr size_t kHeaderBytes = 256;
 constexpr size_t kDoneWord = 1;
 constexpr size_t kTileCounterWord = 16;
-constexpr size_t kSkewWord = 32;  // 16 skewed-place flags of a single sort
+constexpr size_t kRankWordsWord = 32;  // 16 ranking words of a single sort
 
 // Test hooks (onesweep_debug.h), read once per sort when it is planned.
 std::atomic<int64_t> g_fault_tile{-1};
@@ -373,7 +373,7 @@ int run_histogram(const Plan& plan, int key_type, const void* keys, uint64_t n, 
   // the first launch's rows (the first strip's tiles)
   const uint64_t first_tiles = (plan.strip < n ? plan.strip : n + plan.tile - 1) / plan.tile;
   h.clear_words = clear_slab0 ? first_tiles * kRadix : 0;
-  h.skew = reinterpret_cast<uint32_t*>(ws) + kSkewWord;
+  h.rank_words = reinterpret_cast<uint32_t*>(ws) + kRankWordsWord;
   h.top_xor = signed_top_xor(key_type, begin_bit, end_bit, plan.radix_bits);
   h.descending = is_descending(key_type) ? 1u : 0u;
   const int sms = device_sm_count();
@@ -541,7 +541,7 @@ int run_sort(int key_type, const void* keys_in, void* keys_out, const uint32_t* 
       a.error = header;
       a.spin_limit = plan.spin_limit;
       a.fault_tile = plan.fault_tile;
-      a.skew_flags = header + kSkewWord + pass;
+      a.rank_words = header + kRankWordsWord + pass;
       // signed keys: the top place's high digit bit inverted; descending:
       // every digit complemented within its place
       a.digit_xor = (pass == plan.places - 1 ? signed_top_xor(key_type, begin_bit, end_bit, plan.radix_bits) : 0u) ^
@@ -587,7 +587,7 @@ struct BatchPlan {
   uint64_t max_large = 0;    // segments beyond the one-block sorts
   uint64_t max_tiles = 0, max_items = 0;  // capacities (any tile geometry)
   uint64_t grid_tiles = 0;   // tiles at most, with this plan's tile
-  size_t seg_done = 0, seg_hist = 0, zero_end = 0, seg_skew = 0, seg_bin_offsets = 0, large_range = 0, tile_base = 0;
+  size_t seg_done = 0, seg_hist = 0, zero_end = 0, seg_rank_words = 0, seg_bin_offsets = 0, large_range = 0, tile_base = 0;
   size_t hist_base = 0, class_list = 0, hist_large = 0, tile_desc = 0, status[2] = {0, 0};
   size_t alt_keys = 0, alt_vals = 0, total = 0;
 };
@@ -640,7 +640,7 @@ int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int va
   bp->seg_hist = off;
   off = round_up(off + M * per_seg);
   bp->zero_end = off;
-  bp->seg_skew = off;
+  bp->seg_rank_words = off;
   off = round_up(off + M * (size_t)(bp->places > 0 ? bp->places : 1) * 4);
   bp->seg_bin_offsets = off;
   off = round_up(off + M * per_seg);
@@ -742,7 +742,7 @@ int run_batch(int key_type, const void* keys_in, void* keys_out, const uint32_t*
   b.seg_done = reinterpret_cast<uint32_t*>(w + bp.seg_done);
   b.seg_hist = reinterpret_cast<uint32_t*>(w + bp.seg_hist);
   b.seg_bin_offsets = reinterpret_cast<uint32_t*>(w + bp.seg_bin_offsets);
-  b.seg_skew = reinterpret_cast<uint32_t*>(w + bp.seg_skew);
+  b.seg_rank_words = reinterpret_cast<uint32_t*>(w + bp.seg_rank_words);
   b.top_xor = signed_top_xor(key_type, begin_bit, end_bit);
   b.descending = is_descending(key_type) ? 1u : 0u;
   b.error = header;
@@ -797,8 +797,8 @@ int run_batch(int key_type, const void* keys_in, void* keys_out, const uint32_t*
     a.fault_tile = bp.fault_tile;
     a.tile_desc = b.tile_desc;
     a.total_tiles = b.totals;
-    a.skew_flags = b.seg_skew + pass;
-    a.skew_stride = (uint32_t)bp.places;
+    a.rank_words = b.seg_rank_words + pass;
+    a.rank_stride = (uint32_t)bp.places;
     a.digit_xor = (pass == bp.places - 1 ? b.top_xor : 0u) ^ (b.descending ? a.mask : 0u);
     slot = prof_begin(1, pass, s);
     e = launch_binning(bp.key_bits, pairs, bp.cfg, a, s);

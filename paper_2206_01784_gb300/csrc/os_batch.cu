@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kPlanThreads) batch_plan_kernel(BatchArgs b) {
 // and skewed keys cost no more than uniform ones; keys are read with 128-bit
 // streaming loads (the unaligned head and tail of a chunk one key per
 // thread). The flush that completes a segment's items takes the segment's
-// exclusive sums (its bin offsets) and skewed-place flags.
+// exclusive sums (its bin offsets) and ranking words.
 template <int KBITS>
 struct BatchHistLayout {
   static constexpr int P = KBITS / 8;                 // places of 8-bit digits
@@ -172,7 +172,6 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
   constexpr int P = BL::P, C = BL::C;
   constexpr int PER_VEC = 16 / (int)sizeof(K);  // keys per 16-byte vector
   extern __shared__ __align__(16) uint32_t sh[];  // [P * 256][C]
-  __shared__ uint32_t scan_tmp[kSegHistThreads / 32 + 1];
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid & 31;
 
@@ -233,15 +232,10 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
       __threadfence();
       const uint32_t len = __ldcg(b.large_range + seg).y;
       uint32_t* go = b.seg_bin_offsets + (size_t)seg * p * kRadix;
-      for (int pl = 0; pl < p; ++pl) {
-        // descending: bins of the complemented digits (count of t = count of t ^ mask)
-        const uint32_t pmask = pl == p - 1 ? last_mask : 0xFFu;
-        const uint32_t src = b.descending ? (tid ^ pmask) : (uint32_t)tid;
-        const uint32_t c = (tid < kRadix && (uint32_t)tid <= pmask) ? ld_relaxed_gpu(gh + pl * kRadix + src) : 0u;
-        const uint32_t excl = block_exclusive_sum<kSegHistThreads>(c, scan_tmp);
-        if (tid < kRadix) go[pl * kRadix + tid] = excl;
-        const int skewed = __syncthreads_or(tid < kRadix && (uint64_t)c * kSkewDivisor > len);
-        if (tid == 0) b.seg_skew[(size_t)seg * p + pl] = skewed ? 1u : 0u;
+      if (const int pl = tid >> 5; pl < p) {
+        const uint32_t word = finish_place(gh + pl * kRadix, go + pl * kRadix, pl == p - 1 ? last_mask : 0xFFu,
+                                           b.descending, len);
+        if (lane == 0) b.seg_rank_words[(size_t)seg * p + pl] = word;
       }
     }
     __syncthreads();

@@ -88,8 +88,9 @@ template <> struct TileShape<64, 2> { static constexpr int NT = 256, IPT = 8, MI
 // adds one to its digit's counter and reads it back; shared-memory work that
 // slows down when many lanes share a digit).
 constexpr int kRankBallot = 0;    // ballots only
-constexpr int kRankAdaptive = 1;  // counting atomics, or ballots where the pass's place is skewed
+constexpr int kRankAdaptive = 1;  // atomics, one digit apart, or ballots, by the place's ranking word
 constexpr int kRankAtomic = 2;    // counting atomics only
+constexpr int kRankDominant = 3;  // (one digit apart: a body of the adaptive variant, not a variant)
 
 // Batches whose counting atomics are in flight together: they do not depend
 // on one another, so a chunk pays one shared-memory round trip. Pairs keep
@@ -150,7 +151,7 @@ struct TileCtx {
   uint32_t out_base;     // array index of the chain's (segment's) first key
   uint32_t out_len;      // keys in the chain's segment
   uint32_t bulk;         // staged by bulk copies (wait on the mbarriers)
-  uint32_t skewed;       // this place (of this segment) is skewed: rank with ballots only
+  uint32_t rank_word;    // how this place (of this segment) is ranked (rank_word in os_common.cuh)
   const uint32_t* bin_offsets;  // this place's 256 bin offsets (segment-relative)
 };
 
@@ -226,6 +227,26 @@ __device__ __forceinline__ void rank_atomic(uint32_t* cnt, const uint32_t (&d)[U
       if (same) rank[u] = (after[u] & 0xFFFFu) - __popc(peers & lanemask_ge());
       open &= ~peers;
     }
+  }
+}
+
+// Counting atomics with one digit set apart, for a place where many keys share
+// it: their lanes would meet in one counter, one after another, but they are
+// ranked by a single vote, with the digit's running position in a register
+// (`position`, the same in every lane). The other digits then collide little
+// (kRestShares says where that pays).
+template <int U>
+__device__ __forceinline__ void rank_dominant(uint32_t* cnt, uint32_t dominant, uint32_t& position,
+                                              const uint32_t (&d)[U], uint32_t (&rank)[U]) {
+  bool other[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) other[u] = d[u] != dominant;
+  rank_atomic<false, U>(cnt, d, other, rank);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const uint32_t same = __ballot_sync(0xFFFFFFFFu, !other[u]);
+    if (!other[u]) rank[u] = position + __popc(same & lanemask_lt());
+    position += __popc(same);
   }
 }
 
@@ -462,6 +483,8 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
     //     (every key is in registers since the barrier above); for pairs the
     //     positions are kept, two 16-bit positions per register
     uint32_t pos2[PAIRS ? IPT / 2 + 1 : 1];
+    const uint32_t dominant = c.rank_word - 1u;
+    uint32_t dominant_position = RANK == kRankDominant ? wc[dominant] : 0u;
     constexpr int U = RANK == kRankBallot ? 1 : rank_chunk(PAIRS, IPT);
     static_assert(IPT % U == 0 && kRoundEvery % U == 0, "whole chunks of batches");
 #pragma unroll
@@ -472,6 +495,8 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
       for (int u = 0; u < U; ++u) d[u] = digit_of(key[i0 + u], shift, mask, dxor);
       if constexpr (RANK == kRankBallot)
         p[0] = rank_ballot<true, RB>(wc, d[0], true);
+      else if constexpr (RANK == kRankDominant)
+        rank_dominant<U>(wc, dominant, dominant_position, d, p);
       else
         rank_atomic<true, U>(wc, d, valid, p);  // (every lane is valid)
 #pragma unroll
@@ -586,7 +611,7 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
           c.out_base = d.x - local;
           c.out_len = d.y;
           c.bin_offsets = a.bin_offsets + (size_t)d.w * a.offsets_stride;
-          if (RANK == kRankAdaptive && a.skew_flags) c.skewed = a.skew_flags[(size_t)d.w * a.skew_stride];
+          if (RANK == kRankAdaptive && a.rank_words) c.rank_word = a.rank_words[(size_t)d.w * a.rank_stride];
         }
       }
     } else if (tile < a.num_tiles) {
@@ -596,7 +621,7 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
       c.out_base = 0;
       c.out_len = a.out_total;
       c.bin_offsets = a.bin_offsets;
-      if (RANK == kRankAdaptive && a.skew_flags) c.skewed = a.skew_flags[0];
+      if (RANK == kRankAdaptive && a.rank_words) c.rank_word = a.rank_words[0];
     }
     if (c.count > 0 && a.use_bulk) {
       // the 16-byte-aligned span covering the tile, if it stays in the array
@@ -652,12 +677,12 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
       for (uint32_t i = tid; i < c.count; i += NT) vbuf[i] = a.vals_in[c.start + i];
   }
 
-  // adaptive ranking: one uniform branch per tile between two whole bodies
-  // (ballots for a skewed place, counting atomics otherwise)
+  // adaptive ranking: one uniform branch per tile between whole bodies
   constexpr int R0 = RANK == kRankAdaptive ? kRankAtomic : RANK;
-  const bool ballots = RANK == kRankAdaptive && c.skewed;
-  if (ballots)
+  if (RANK == kRankAdaptive && c.rank_word == kRankWordBallots)
     binning_tile<KBITS, PAIRS, CFG, kRankBallot, FLIP, RB>(a, smem, c);
+  else if (RANK == kRankAdaptive && c.rank_word != 0u)
+    binning_tile<KBITS, PAIRS, CFG, kRankDominant, FLIP, RB>(a, smem, c);
   else
     binning_tile<KBITS, PAIRS, CFG, R0, FLIP, RB>(a, smem, c);
 }

@@ -425,7 +425,7 @@ __device__ void ws_rankers(const PassArgs& a, unsigned char* smem) {
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::bars);
   const WsTile* sctx = reinterpret_cast<const WsTile*>(smem + C::ctx);
   constexpr int R1 = RANK == kRankBallot ? kRankBallot : kRankAtomic;
-  const bool ballots = RANK == kRankBallot || (RANK == kRankAdaptive && a.skew_flags && *a.skew_flags);
+  const bool ballots = RANK == kRankBallot || (RANK == kRankAdaptive && a.rank_words && *a.rank_words != 0u);
 
   // thread 0 stages the first tile and takes the id of the second
   uint32_t next = 0;
@@ -450,7 +450,7 @@ __device__ void ws_rankers(const PassArgs& a, unsigned char* smem) {
       return;
     }
     // one uniform branch per tile between whole tile bodies: ballots only
-    // (a skewed place, or the ballot variant) or the counting atomics
+    // (a place that is not ranked by atomics alone, or the ballot variant) or the counting atomics
     bool stop = false;
     if (t.count == (uint32_t)C::T) {
       if (ballots)

@@ -29,9 +29,22 @@ constexpr uint32_t kAggSpanShift = 24;
 constexpr uint32_t kAggValueMask = (1u << kAggSpanShift) - 1u;
 constexpr uint32_t kAggMaxSpan = 64;
 
-// A digit place is skewed (its binning pass ranks with ballots only) when one
-// digit holds more than 1/kSkewDivisor of the keys.
-constexpr uint32_t kSkewDivisor = 8;
+// How a binning pass ranks a place's digits, by what the place's histogram says
+// of the 496 pairs of lanes in a batch: with counting atomics while few pairs
+// share a digit (the sum of the squared shares of all digits is up to
+// kAtomicShares); with the most frequent digit apart while few pairs share one
+// of the others (up to kRestShares); else with ballots, which do not slow down
+// when lanes share digits. Measured at 2^26 u32 pairs / keys only, us a sort;
+// keys that are the AND of q uniform words, sums of all / all but the first:
+//   uniform .004 / .004   atomics 1120 / 770    ballots 1428 / -
+//   q = 2   .023 / .013   apart 1390 / 1090     ballots 1440 / 1199, atomics 1459 / 1170
+//   q = 3   .138 / .020   apart 1486 / 1213     ballots 1410 / 1192, atomics 1823 / 1567
+//   q = 5   .605 / .005   apart 1160 / 907      ballots 1339 / 1158
+//   q = 8   .939 / .000   apart 1061 / -        ballots 1303 / -
+constexpr float kAtomicShares = 0.018f;
+constexpr float kRestShares = 0.016f;
+// A place's ranking word: 0 atomics, 1 + digit that digit apart, kRankWordBallots.
+constexpr uint32_t kRankWordBallots = 0xFFFFu;
 
 // Bits of the workspace's device status word.
 constexpr uint32_t kErrTimeout = 1u;
@@ -153,36 +166,56 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// ---------------------------------------------------------------- block scan
+// ---------------------------------------------------------------- one place
 
-// Exclusive prefix sum over the NT threads of a block (each contributes v).
-// `tmp` holds NT/32 + 1 words of shared memory. Contains __syncthreads().
-template <int NT>
-__device__ __forceinline__ uint32_t block_exclusive_sum(uint32_t v, uint32_t* tmp, uint32_t* total = nullptr) {
-  constexpr int NW = NT / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t x = v;
+// Called by a whole warp once a place's counts are complete (in `hist`, read
+// past L1): writes the exclusive sums of its 256 bins to `offsets` and returns
+// its ranking word (in every lane). last_digit: the place's highest digit. A
+// descending sort bins by the complement of each digit within its place - the
+// count of complemented digit t is the count of digit t ^ last_digit - and
+// `hist` is then rewritten in that order. One warp per place and no block
+// barrier: the places' sums are taken side by side by the block that completes
+// the counts, while every other block waits for the next launch.
+__device__ __forceinline__ uint32_t finish_place(uint32_t* hist, uint32_t* offsets, uint32_t last_digit,
+                                                 bool descending, uint64_t n) {
+  constexpr int PER = kRadix / 32;  // bins of a lane
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t c[PER], sum = 0, most = 0;
+  float shares = 0.0f;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const uint32_t d = lane * PER + j;
+    c[j] = d <= last_digit ? ld_relaxed_gpu(hist + (descending ? d ^ last_digit : d)) : 0u;
+  }
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const float p = (float)c[j] / (float)n;
+    shares += p * p;
+    sum += c[j];
+    most = max(most, c[j]);
+  }
+  uint32_t incl = sum;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    if (lane >= o) incl += y;
+    shares += __shfl_xor_sync(0xFFFFFFFFu, shares, o);
   }
-  if (lane == 31) tmp[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t w = lane < NW ? tmp[lane] : 0u;
-    uint32_t s = w;
+  uint32_t run = incl - sum;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-      if (lane >= o) s += y;
-    }
-    if (lane < NW) tmp[lane] = s - w;
-    if (lane == NW - 1) tmp[NW] = s;
+  for (int j = 0; j < PER; ++j) {
+    offsets[lane * PER + j] = run;
+    run += c[j];
+    if (descending) hist[lane * PER + j] = c[j];  // (every lane has read, by the shuffles above)
   }
-  __syncthreads();
-  if (total) *total = tmp[NW];
-  return tmp[warp] + x - v;
+  const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, most);
+  uint32_t digit = kRadix;
+#pragma unroll
+  for (int j = PER - 1; j >= 0; --j)
+    if (c[j] == top) digit = lane * PER + j;
+  digit = __reduce_min_sync(0xFFFFFFFFu, digit);
+  const float p = (float)top / (float)n;
+  return shares <= kAtomicShares ? 0u : shares - p * p <= kRestShares ? 1u + digit : kRankWordBallots;
 }
 
 }  // namespace onesweep

@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(kHistThreads, 1) histogram_kernel(HistArgs a) 
   constexpr int PER_VEC = 128 / KBITS;     // keys per 16-byte vector
   constexpr int KPT = kHistVec * PER_VEC;  // keys per thread per step
   extern __shared__ __align__(16) uint32_t sh[];  // [P * 256][kCopies]
-  __shared__ uint32_t scan_tmp[kHistThreads / 32 + 1];
   __shared__ uint32_t s_last;
 
   const int tid = threadIdx.x;
@@ -188,22 +187,11 @@ __global__ void __launch_bounds__(kHistThreads, 1) histogram_kernel(HistArgs a) 
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int pl = 0; pl < p; ++pl) {
-    // a descending sort bins by the complement of each digit within its
-    // place: count of complemented digit t = count of digit t ^ mask
-    const uint32_t pmask = pl == p - 1 ? last_mask : (uint32_t)nbin - 1u;
-    const uint32_t src = a.descending ? (tid ^ pmask) : (uint32_t)tid;
-    const uint32_t c = (tid < kRadix && (uint32_t)tid <= pmask) ? ld_relaxed_gpu(a.hist + pl * kRadix + src) : 0u;
-    const uint32_t excl = block_exclusive_sum<kHistThreads>(c, scan_tmp);
-    if (tid < kRadix) a.offsets[pl * kRadix + tid] = excl;
-    // (every read of this place's counts is before the scan's barriers)
-    if (a.descending && tid < kRadix) a.hist[pl * kRadix + tid] = c;
-    // a place where one digit holds over 1/8 of the keys is "skewed": its
-    // binning pass ranks with ballots, which do not slow down when many lanes
-    // share a digit (measured on GB300: at ~10 % in one digit the lane masks
-    // are still faster, at ~34 % the ballots are)
-    const int skewed = __syncthreads_or(tid < kRadix && (uint64_t)c * kSkewDivisor > a.n);
-    if (tid == 0 && a.skew) a.skew[pl] = skewed ? 1u : 0u;
+  static_assert(L::kMaxP + 1 <= kHistThreads / 32, "one warp per place");
+  if (const int pl = tid >> 5; pl < p) {
+    const uint32_t word = finish_place(a.hist + pl * kRadix, a.offsets + pl * kRadix,
+                                       pl == p - 1 ? last_mask : (uint32_t)nbin - 1u, a.descending, a.n);
+    if ((tid & 31) == 0 && a.rank_words) a.rank_words[pl] = word;
   }
 }
 

@@ -40,7 +40,7 @@ struct HistArgs {
   uint32_t* done_counter;    // zeroed by the caller (device)
   uint32_t* clear;           // words to zero on the way (status slab of pass 0), may be null
   uint64_t clear_words;
-  uint32_t* skew;            // [p] set to 1 where one digit holds over 1/16 of the keys (may be null)
+  uint32_t* rank_words;      // [p] how each place's digits are ranked (rank_word; may be null)
   uint32_t top_xor;          // signed keys: high bit of the top place's digit inverted (else 0)
   uint32_t descending;       // offsets (and the reported histograms) for complemented digits
 };
@@ -80,15 +80,15 @@ struct PassArgs {
   // keys. Each large segment is its own sort: its tiles form one look-back
   // chain and it has its own bin offsets. A tile's descriptor: array index of
   // its first key, its segment's length, its chain's first tile, its segment's
-  // row (bin offsets, skew flags).
+  // row (bin offsets, ranking words).
   const uint4* tile_desc;        // [tiles]
   const uint32_t* total_tiles;   // device word: tiles in this pass
   uint32_t offsets_stride;       // words between two segments' bin offsets
 
-  // Skewed-place flags from the histogram pass (null: none); the flag of
-  // segment s (0 for one array) is skew_flags[s * skew_stride].
-  const uint32_t* skew_flags;
-  uint32_t skew_stride;
+  // Ranking words from the histogram pass (null: none); the word of segment s
+  // (0 for one array) is rank_words[s * rank_stride].
+  const uint32_t* rank_words;
+  uint32_t rank_stride;
   uint32_t digit_xor;            // signed keys, top place: invert the digit's high bit (else 0)
 };
 
@@ -153,7 +153,7 @@ struct BatchArgs {
   uint32_t* seg_done;            // [max_large] zeroed
   uint32_t* seg_hist;            // [max_large][p][256] zeroed
   uint32_t* seg_bin_offsets;     // [max_large][p][256]
-  uint32_t* seg_skew;            // [max_large][p] skewed-place flags
+  uint32_t* seg_rank_words;      // [max_large][p]
   uint32_t top_xor;              // signed keys: high bit of the top place's digit inverted (else 0)
   uint32_t descending;           // bin by the complemented digit of every place
   uint32_t* error;
