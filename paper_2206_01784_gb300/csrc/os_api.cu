@@ -551,6 +551,7 @@ int run_sort(int key_type, const void* keys_in, void* keys_out, const uint32_t* 
         return OS_ERR_INVALID_ARG;
       }
       const int slot = prof_begin(1, pass, s);
+      a.early = slot < 0;  // (not with an event in between)
       const cudaError_t e = launch_binning(plan.key_bits, pairs, plan.cfg, a, s, plan.radix_bits);
       prof_end(slot, s);
       if (e != cudaSuccess) return OS_ERR_CUDA;
@@ -801,6 +802,7 @@ int run_batch(int key_type, const void* keys_in, void* keys_out, const uint32_t*
     a.rank_stride = (uint32_t)bp.places;
     a.digit_xor = (pass == bp.places - 1 ? b.top_xor : 0u) ^ (b.descending ? a.mask : 0u);
     slot = prof_begin(1, pass, s);
+    a.early = slot < 0;  // (not with an event in between)
     e = launch_binning(bp.key_bits, pairs, bp.cfg, a, s);
     prof_end(slot, s);
     if (e != cudaSuccess) return OS_ERR_CUDA;

@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
   extern __shared__ __align__(16) uint32_t sh[];  // [P * 256][C]
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x, lane = tid & 31;
+  pdl_launch_dependents();
 
   {
     uint4* s4 = reinterpret_cast<uint4*>(sh);

@@ -380,7 +380,7 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   // the next pass's status counters of this tile start at N
   if (a.status_clear && tid < kRadix)
     for (size_t row = tile; row < a.status_clear_rows; row += a.num_tiles) a.status_clear[row * kRadix + tid] = 0u;
-  const uint32_t bin_offset = tid < R ? __ldg(c.bin_offsets + tid) : 0u;
+  const uint32_t bin_offset = tid < R ? c.bin_offsets[tid] : 0u;
   uint32_t* status = a.status + (size_t)tile * kRadix;
   const bool publish = (int64_t)tile != a.fault_tile;
   const bool chain_head = tile == c.chain_first;
@@ -594,9 +594,13 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
   __shared__ TileCtx s_ctx;
   const int tid = threadIdx.x;
 
-  // 1. tile id and where the tile sits
+  // 1. tile id and where the tile sits. The launch may start while the one
+  // before it ends (programmatic dependent launch): only the tile id, from a
+  // counter that no other launch touches, is taken before the wait for it.
+  uint32_t tile = 0;
+  if (tid == 0) tile = atomicAdd(a.tile_counter, 1u);
+  pdl_wait();
   if (tid == 0) {
-    const uint32_t tile = atomicAdd(a.tile_counter, 1u);
     TileCtx c{};
     c.tile = tile;
     if (SEG) {
@@ -667,6 +671,7 @@ __global__ void __launch_bounds__(BinningConfig<KBITS, PAIRS, CFG>::NT, BinningC
   }
   __syncthreads();
   const TileCtx c = s_ctx;
+  pdl_launch_dependents();  // the next launch's blocks may take the slots that this one's last blocks leave
   if (c.count == 0) return;  // no tile left (or the workspace's counters were not reset)
 
   // 2. plain staging when the bulk copy does not apply

@@ -619,8 +619,8 @@ cudaError_t launch_binning_one(const PassArgs& a, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(binning_kernel<KBITS, PAIRS, CFG, RANK, FLIP, SEG, RB>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_bytes);
   if (e != cudaSuccess) return e;
-  binning_kernel<KBITS, PAIRS, CFG, RANK, FLIP, SEG, RB><<<a.num_tiles, C::NT, C::smem_bytes, s>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(binning_kernel<KBITS, PAIRS, CFG, RANK, FLIP, SEG, RB>, a.num_tiles, C::NT, C::smem_bytes, s,
+                       a.early != 0u, a);
 }
 
 // Digits narrower than 8 bits (the digit-width sweep of Section 4, Table 2):

@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kHistThreads, 1) histogram_kernel(HistArgs a) 
 
   const int tid = threadIdx.x;
   const int p = a.num_places;
+  pdl_launch_dependents();
   {
     uint4* s4 = reinterpret_cast<uint4*>(sh);
     for (int i = tid; i < L::kEntries * C / 4; i += kHistThreads) s4[i] = make_uint4(0, 0, 0, 0);

@@ -9,7 +9,11 @@
 namespace onesweep {
 
 // Launches a one-argument kernel; early: it may start once every block of the
-// stream's last kernel has called pdl_launch_dependents or has ended.
+// stream's last kernel has called pdl_launch_dependents or has ended. Between
+// the passes of a sort that hides the launch, the first tile ids and the last
+// blocks' drain: 3.3M u32 keys 78 -> 68 us, 2.0M u64 pairs 161 -> 141, 2^28 u32
+// pairs 4218 -> 4180. (A proxy fence before the bulk copies, which the wait
+// does not need, made every pass 5 % slower.)
 template <typename Args>
 cudaError_t launch_kernel(void (*kernel)(Args), unsigned grid, unsigned threads, size_t smem_bytes, cudaStream_t s,
                           bool early, const Args& args) {
@@ -90,6 +94,7 @@ struct PassArgs {
   const uint32_t* rank_words;
   uint32_t rank_stride;
   uint32_t digit_xor;            // signed keys, top place: invert the digit's high bit (else 0)
+  uint32_t early;                // may start while the stream's last kernel, of this library, ends
 };
 
 // A whole sort in one launch (os_small.cu).
