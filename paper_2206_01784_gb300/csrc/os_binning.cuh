@@ -30,7 +30,7 @@
 //     replaced by lane order (rank_atomic). With counters that start at local
 //     positions, the rank is the key's place in the tile's shared-memory
 //     bins, and the key is written there at once.
-//     Every kRoundEvery batches the look-back's round in flight is folded in
+//     Every few batches the look-back's round in flight is folded in
 //     and the next one sent, so its L2 round trips ride along the ranking. A
 //     __match_any_sync per key measured 1.7x slower than the ballots on
 //     GB300 (the match instruction saturates the ADU pipe) and is not used;
@@ -340,17 +340,26 @@ struct Lookback {
     if (!done) publish_global();
   }
 };
-constexpr int kLookbackWindow = 4;
+// Counters read per look-back round. A walk is rarely long - a tile's
+// predecessors have mostly published spans or prefixes - and every further
+// counter of a round costs registers, issue slots and L2 reads in all 256
+// walkers. 2^28 u32 pairs / keys only, us a sort, with 8, 6, 4, 3, 2 and 1
+// counters (8, 6 and 3 in a build 1.5 / 3 % slower): 4432 / 3285, 4348 / 3223,
+// 4212 / 3077, 4231 / 3121, 4104 / 3007, 4102 / 2998.
+constexpr int kLookbackWindow = 1;
 // Tiles ahead whose keys (and values) a starting block prefetches into L2
 // (measured at 2^28 keys on GB300: 48, 144 and 384 tiles ahead all shorten a
 // pass by about 1 %; the tile's own staging copy then waits less).
 constexpr uint32_t kPrefetchTiles = 48;
 // Ranking batches between two look-back rounds: about one L2 round trip of
-// ranking work, so a round's reads have come back when it is consumed.
-#ifndef OS_ROUND_EVERY
-#define OS_ROUND_EVERY 8
-#endif
-constexpr int kRoundEvery = OS_ROUND_EVERY;
+// ranking work, so a round's reads have come back when it is consumed. With one
+// counter a round, keys only rank fast enough for a round every 4 batches (2^28
+// u32 keys 2949 us a sort, every 8 2998; 2^26 u64 keys 2338, 2361); pairs and
+// the other ranking methods do not (2^28 u32 pairs 4100, 4102; 2^26 pairs of 3-
+// word keys 1398, 1361, 5-word keys 1143, 1114).
+__host__ __device__ constexpr int round_every(bool pairs, int rank) {
+  return !pairs && rank == kRankAtomic ? 4 : 8;
+}
 
 template <int KBITS, bool PAIRS, int CFG, int RANK, int FLIP, int RB>
 __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* smem, const TileCtx& c) {
@@ -486,7 +495,8 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
     const uint32_t dominant = c.rank_word - 1u;
     uint32_t dominant_position = RANK == kRankDominant ? wc[dominant] : 0u;
     constexpr int U = RANK == kRankBallot ? 1 : rank_chunk(PAIRS, IPT);
-    static_assert(IPT % U == 0 && kRoundEvery % U == 0, "whole chunks of batches");
+    constexpr int kRound = round_every(PAIRS, RANK);
+    static_assert(IPT % U == 0 && kRound % U == 0, "whole chunks of batches");
 #pragma unroll
     for (int i0 = 0; i0 < IPT; i0 += U) {
       uint32_t d[U], p[U];
@@ -511,7 +521,7 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
         }
       }
       // a look-back round: fold in the last one's reads, send the next
-      if ((i0 + U) % kRoundEvery == 0 && i0 + U < IPT && walker) {
+      if ((i0 + U) % kRound == 0 && i0 + U < IPT && walker) {
         if (issued) lb.consume();
         issued = !lb.done;
         if (issued) lb.issue(a.status, c.chain_first, tid);
