@@ -51,23 +51,26 @@ __device__ __forceinline__ void unpack<64>(const uint4& v, uint64_t* out) {
   out[1] = ((uint64_t)v.w << 32) | v.z;
 }
 
-// FULL: the sort covers every key bit ([0, KBITS): all places 8 bits wide,
-// digit i = byte i), so a digit is one shift and mask. FLIP: float keys (the
+// RB: the sort covers every key bit in digits of RB bits, so a digit is one
+// shift and mask; 0: any bit range and digit width. FLIP: float keys (the
 // sign-flip before counting). Both are compile-time so the counting loop, the
 // kernel's whole cost (one shared-memory atomic per key and place, the issue
-// slots around it), carries no per-key branches.
-template <int KBITS, bool FULL, bool FLIP>
+// slots around it), carries no per-key branches. With the width known here,
+// against the body for any range, us: 2^28 u32 keys 243 / 603 in 5-bit digits,
+// 216 / 528 in 6, 188 / 455 in 7, 174 in 8; 2^26 u64 keys 203 / 708, 176 / 611,
+// 157 / 555, 137 (the reading alone takes 158 and 79 at 6.8 TB/s).
+template <int KBITS, int RB, bool FLIP>
 __global__ void __launch_bounds__(kHistThreads, 1) histogram_kernel(HistArgs a) {
   using K = typename KeyWord<KBITS>::type;
   using L = HistLayout<KBITS>;
-  constexpr int P = L::P, C = L::kCopies;
+  constexpr int P = RB ? (KBITS + RB - 1) / RB : L::kMaxP + 1, C = L::kCopies;
   constexpr int PER_VEC = 128 / KBITS;     // keys per 16-byte vector
   constexpr int KPT = kHistVec * PER_VEC;  // keys per thread per step
   extern __shared__ __align__(16) uint32_t sh[];  // [P * 256][kCopies]
   __shared__ uint32_t s_last;
 
   const int tid = threadIdx.x;
-  const int p = a.num_places;
+  const int p = RB ? P : a.num_places;
   pdl_launch_dependents();
   {
     uint4* s4 = reinterpret_cast<uint4*>(sh);
@@ -83,30 +86,23 @@ __global__ void __launch_bounds__(kHistThreads, 1) histogram_kernel(HistArgs a) 
   }
   __syncthreads();
 
-  // digits of rb bits (8 in the FULL mode): place i covers bits
+  // digits of rb bits: place i covers bits
   // [begin + rb*i, +rb), the last one possibly narrower; counter (place,
   // digit) of this lane's copy at word ((place * 2^rb + digit) * C + copy)
-  const int rb = FULL ? 8 : a.radix_bits;
+  const int rb = RB ? RB : a.radix_bits;
   const int nbin = 1 << rb;
-  const uint32_t last_mask = (1u << (a.end_bit - (a.begin_bit + rb * (p - 1)))) - 1u;
+  const int begin_bit = RB ? 0 : a.begin_bit, end_bit = RB ? KBITS : a.end_bit;
+  const uint32_t last_mask = (1u << (end_bit - (begin_bit + rb * (p - 1)))) - 1u;
   uint32_t* mine = sh + (tid & 31) % C;
   const uint32_t top_xor = a.top_xor;
   auto count_key = [&](K k) {
     const K o = FLIP ? flip_to_ordered(k) : k;
-    if (FULL) {
 #pragma unroll
-      for (int pl = 0; pl < P; ++pl) {
-        const uint32_t d = (uint32_t)(o >> (8 * pl)) & 0xFFu;
-        atomicAdd(mine + (pl * kRadix + (pl == P - 1 ? d ^ top_xor : d)) * C, 1u);
-      }
-    } else {
-#pragma unroll
-      for (int pl = 0; pl < L::kMaxP + 1; ++pl) {
-        if (pl < p) {
-          const uint32_t d = digit_of(o, a.begin_bit + rb * pl, pl == p - 1 ? last_mask : (uint32_t)nbin - 1u,
-                                      pl == p - 1 ? top_xor : 0u);
-          atomicAdd(mine + (pl * nbin + d) * C, 1u);
-        }
+    for (int pl = 0; pl < P; ++pl) {
+      if (RB || pl < p) {
+        const uint32_t d = digit_of(o, begin_bit + rb * pl, pl == p - 1 ? last_mask : (uint32_t)nbin - 1u,
+                                    pl == p - 1 ? top_xor : 0u);
+        atomicAdd(mine + (pl * nbin + d) * C, 1u);
       }
     }
   };
@@ -196,23 +192,33 @@ __global__ void __launch_bounds__(kHistThreads, 1) histogram_kernel(HistArgs a) 
   }
 }
 
-template <int KBITS, bool FULL, bool FLIP>
+template <int KBITS, int RB, bool FLIP>
 cudaError_t launch_hist_mode(const HistArgs& a, int grid, cudaStream_t s) {
   constexpr size_t bytes = HistLayout<KBITS>::smem_bytes;
   // set on every launch: an idempotent host-side attribute, so concurrent
   // callers on any device need no shared state
-  cudaError_t e = cudaFuncSetAttribute(histogram_kernel<KBITS, FULL, FLIP>,
+  cudaError_t e = cudaFuncSetAttribute(histogram_kernel<KBITS, RB, FLIP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  histogram_kernel<KBITS, FULL, FLIP><<<grid, kHistThreads, bytes, s>>>(a);
+  histogram_kernel<KBITS, RB, FLIP><<<grid, kHistThreads, bytes, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int KBITS, int RB>
+cudaError_t launch_hist_flip(const HistArgs& a, int grid, cudaStream_t s) {
+  return a.flip ? launch_hist_mode<KBITS, RB, true>(a, grid, s) : launch_hist_mode<KBITS, RB, false>(a, grid, s);
 }
 
 template <int KBITS>
 cudaError_t launch_hist_t(const HistArgs& a, int grid, cudaStream_t s) {
-  const bool full = a.begin_bit == 0 && a.end_bit == KBITS && a.num_places == KBITS / 8 && a.radix_bits == 8;
-  if (full) return a.flip ? launch_hist_mode<KBITS, true, true>(a, grid, s) : launch_hist_mode<KBITS, true, false>(a, grid, s);
-  return a.flip ? launch_hist_mode<KBITS, false, true>(a, grid, s) : launch_hist_mode<KBITS, false, false>(a, grid, s);
+  const bool full = a.begin_bit == 0 && a.end_bit == KBITS && a.num_places == (KBITS + a.radix_bits - 1) / a.radix_bits;
+  switch (full ? a.radix_bits : 0) {
+    case 5: return launch_hist_flip<KBITS, 5>(a, grid, s);
+    case 6: return launch_hist_flip<KBITS, 6>(a, grid, s);
+    case 7: return launch_hist_flip<KBITS, 7>(a, grid, s);
+    case 8: return launch_hist_flip<KBITS, 8>(a, grid, s);
+    default: return launch_hist_flip<KBITS, 0>(a, grid, s);
+  }
 }
 
 }  // namespace
@@ -237,7 +243,7 @@ cudaError_t launch_histogram(int key_bits, const HistArgs& a, int num_sms, cudaS
 // sm_103a), or a negative CUDA error code.
 extern "C" OS_API int os_binary_version(void) {
   cudaFuncAttributes fa{};
-  const cudaError_t e = cudaFuncGetAttributes(&fa, onesweep::histogram_kernel<32, true, false>);
+  const cudaError_t e = cudaFuncGetAttributes(&fa, onesweep::histogram_kernel<32, 8, false>);
   return e == cudaSuccess ? fa.binaryVersion : -(int)e;
 }
 
