@@ -351,6 +351,13 @@ constexpr int kLookbackWindow = 1;
 // (measured at 2^28 keys on GB300: 48, 144 and 384 tiles ahead all shorten a
 // pass by about 1 %; the tile's own staging copy then waits less).
 constexpr uint32_t kPrefetchTiles = 48;
+// Keys a thread writes per step of the write-out. Nothing there has to stay in
+// registers, and a body unrolled whole spends its time on instruction fetches
+// (ncu: 12 % of the warps' stalls). us a sort, unrolled by 32 / 4 / 2 / 1: 2^28
+// u32 pairs 4100 / 4064 / 4004 / 4112, keys only 2940 / 2907 / 2953 / 3128; 2^26
+// u64 pairs 2964 / 2938 / 2945 / 3038; 2^26 pairs of 2-word keys 1344 / 1298 /
+// 1275 / 1319; 3.3M u32 pairs 87.3 / 85.2 / 87.2 / 87.4.
+constexpr int kWriteUnroll = 4;
 // Ranking batches between two look-back rounds: about one L2 round trip of
 // ranking work, so a round's reads have come back when it is consumed. With one
 // counter a round, keys only rank fast enough for a round every 4 batches (2^28
@@ -572,7 +579,7 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
       }
     }
   } else {
-#pragma unroll
+#pragma unroll kWriteUnroll
     for (int i = 0; i < IPT; ++i) {
       const uint32_t j = i * NT + tid;
       const K k = kt[j];
