@@ -79,12 +79,15 @@ constexpr int kTileConfigs = 3 * kGeometries;
 // os_set_tile_config / os_set_tile_config_bucket (the autotuner's hooks) and
 // read once per sort when it is planned, with atomic loads and stores (a
 // sort may also name its variant itself: os_sort_*_ex).
-// Default everywhere: geometry 0 with adaptive ranking, the fastest measured
-// on GB300 for 32- and 64-bit keys from 2^21 keys up (64-bit pairs at 2^27:
-// 0.714 ms per pass against 0.929 with the persistent geometry).
+// Default everywhere: adaptive ranking, the tile by size (make_plan,
+// make_batch_plan); from 2^22 keys up geometry 0 is the fastest measured on
+// GB300 (64-bit pairs at 2^27: 0.714 ms per pass against 0.929 with the
+// persistent geometry).
 constexpr int kDefaultTileConfig = kGeometries + 0;
+constexpr int kSms = 152;  // of a GB300 (the lines between tile geometries; nothing else depends on it)
 constexpr int kSizeBuckets = 4;  // n < 2^16, < 2^20, < 2^24, larger
-#define OS_FOUR_DEFAULTS {kDefaultTileConfig, kDefaultTileConfig, kDefaultTileConfig, kDefaultTileConfig}
+constexpr int kNotSet = -1;  // the default variant, its tile by size
+#define OS_FOUR_DEFAULTS {kNotSet, kNotSet, kNotSet, kNotSet}
 int g_tile_cfg[2][2][kSizeBuckets] = {{OS_FOUR_DEFAULTS, OS_FOUR_DEFAULTS}, {OS_FOUR_DEFAULTS, OS_FOUR_DEFAULTS}};
 #undef OS_FOUR_DEFAULTS
 
@@ -98,8 +101,12 @@ int get_radix_bits(int key_bits, bool pairs, int bucket) {
   return v == 0 ? kRadixBits : v;
 }
 
-int get_tile_cfg(int key_bits, bool pairs, int bucket) {
+int raw_tile_cfg(int key_bits, bool pairs, int bucket) {
   return __atomic_load_n(&g_tile_cfg[key_bits == 64][pairs][bucket], __ATOMIC_RELAXED);
+}
+int get_tile_cfg(int key_bits, bool pairs, int bucket) {
+  const int cfg = raw_tile_cfg(key_bits, pairs, bucket);
+  return cfg == kNotSet ? kDefaultTileConfig : cfg;
 }
 void set_tile_cfg(int key_bits, bool pairs, int bucket, int cfg) {
   __atomic_store_n(&g_tile_cfg[key_bits == 64][pairs][bucket], cfg, __ATOMIC_RELAXED);
@@ -267,10 +274,27 @@ int make_plan(int key_type, uint64_t n, int value_bytes, int begin_bit, int end_
   plan->bucket = size_bucket(n);
   // the variant is read once: every launch of this sort uses the same one
   if (cfg_override >= kTileConfigs) return OS_ERR_INVALID_ARG;
-  plan->cfg = cfg_override >= 0 ? cfg_override : binning_config(kb, plan->pairs, plan->bucket);
+  const int set_cfg = cfg_override >= 0 ? cfg_override : raw_tile_cfg(kb, plan->pairs, plan->bucket);
+  plan->cfg = set_cfg == kNotSet ? kDefaultTileConfig : set_cfg;
   if (radix_bits != kRadixBits) {
     if (cfg_override >= 0 && cfg_override != kGeometries) return OS_ERR_INVALID_ARG;
     plan->cfg = kGeometries;  // geometry 0, adaptive ranking
+  }
+  // The default variant takes smaller tiles while these make one wave of blocks
+  // (geometry 2: 4 an SM, geometry 1: 3): a pass then takes as long as a tile.
+  // us a sort with geometry 0 / 1 / 2, in brackets of 13 key bits: u32 pairs, 1.9M keys 82 / 70 / 68 (52 / 46 / 44), 2.5M 84 /
+  // 73 / 79 (54 / 47 / 48), 3.0M 85 / 99 / 100, 4.2M 121 / 114 / 113, 5.0M 132 /
+  // 124 / 131 (of skewed i32 keys, with cold inputs, 156 / 159), 6.5M 152 / 158 / 163; u32 keys, 1.9M 61 / 55 / 56, 3.0M 65 / 80 /
+  // 82, 5.0M 102 / 93 / 99; u64 pairs, 1.3M 136 / 123 / 126, 2.0M 140 / 175 /
+  // 176, 2.4M 178 / 191 / 191; u64 keys, 1.3M 107 / 100 / 105, 2.4M 145 / 158 /
+  // 160, 3.0M 177 / 169 / 202.
+  if (set_cfg == kNotSet && radix_bits == kRadixBits) {
+    const uint64_t wave1 = 3ull * kSms * tile_keys_for(kb, plan->pairs, kDefaultTileConfig + 1);
+    const uint64_t wave2 = 4ull * kSms * tile_keys_for(kb, plan->pairs, kDefaultTileConfig + 2);
+    if (n <= wave2)
+      plan->cfg += 2;
+    else if (n <= wave1)
+      plan->cfg += 1;
   }
   plan->fault_tile = g_fault_tile.load(std::memory_order_relaxed);
   plan->spin_limit = g_spin_limit.load(std::memory_order_relaxed);

@@ -302,17 +302,19 @@ __global__ void __launch_bounds__(kSegHistThreads, 1) batch_histogram_kernel(Bat
 // (programmatic dependent launch) and fills the SMs that it leaves idle. Block 0
 // waits for the kernel before to complete before it ends itself: what the
 // stream runs after the last of them then follows them all.
-template <int KBITS, bool PAIRS, int CLS>
+template <int KBITS, bool PAIRS, int CLS, bool WIDE>
 struct ClassTile {
-  static constexpr BatchClass kClass = KBITS == 32 ? kClass32[CLS] : kClass64[CLS];
+  static constexpr BatchClass kShape = KBITS == 32 ? kClass32[CLS] : kClass64[CLS];
+  static constexpr BatchClass kClass = WIDE ? BatchClass{1024, (int)kShape.capacity() / 1024, 1} : kShape;
   using Tile = SmallTile<KBITS, PAIRS, kClass.threads, kClass.keys_per_thread, true, true>;
   static_assert(kClass.blocks_per_sm * (Tile::smem_bytes + 1024) <= 228 * 1024, "blocks of a class on an SM");
 };
 
-template <int KBITS, bool PAIRS, int CLS>
-__global__ void __launch_bounds__(ClassTile<KBITS, PAIRS, CLS>::kClass.threads, ClassTile<KBITS, PAIRS, CLS>::kClass.blocks_per_sm)
+template <int KBITS, bool PAIRS, int CLS, bool WIDE>
+__global__ void __launch_bounds__(ClassTile<KBITS, PAIRS, CLS, WIDE>::kClass.threads,
+                                  ClassTile<KBITS, PAIRS, CLS, WIDE>::kClass.blocks_per_sm)
     batch_class_sort_kernel(BatchArgs b) {
-  using Tile = typename ClassTile<KBITS, PAIRS, CLS>::Tile;
+  using Tile = typename ClassTile<KBITS, PAIRS, CLS, WIDE>::Tile;
   using K = typename Tile::K;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint32_t s_item;
@@ -338,10 +340,10 @@ __global__ void __launch_bounds__(ClassTile<KBITS, PAIRS, CLS>::kClass.threads, 
   if (blockIdx.x == 0) pdl_wait();
 }
 
-template <int KBITS, bool PAIRS, int CLS>
+template <int KBITS, bool PAIRS, int CLS, bool WIDE>
 cudaError_t launch_class(const BatchArgs& b, bool* after_kernel, cudaStream_t s) {
-  using CT = ClassTile<KBITS, PAIRS, CLS>;
-  auto* kernel = batch_class_sort_kernel<KBITS, PAIRS, CLS>;
+  using CT = ClassTile<KBITS, PAIRS, CLS, WIDE>;
+  auto* kernel = batch_class_sort_kernel<KBITS, PAIRS, CLS, WIDE>;
   // set on every launch: an idempotent host-side attribute
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CT::Tile::smem_bytes);
   if (e != cudaSuccess) return e;
@@ -361,9 +363,16 @@ cudaError_t launch_class(const BatchArgs& b, bool* after_kernel, cudaStream_t s)
 // first of them waits for the plan as any kernel does.
 template <int KBITS, bool PAIRS>
 cudaError_t launch_classes(const BatchArgs& b, bool* after_class, cudaStream_t s) {
-  cudaError_t e = launch_class<KBITS, PAIRS, 2>(b, after_class, s);
-  if (e == cudaSuccess) e = launch_class<KBITS, PAIRS, 1>(b, after_class, s);
-  if (e == cudaSuccess) e = launch_class<KBITS, PAIRS, 0>(b, after_class, s);
+  // few segments: every SM has one or two, whose own time counts, so a segment
+  // gets a whole block of 1024 threads (us a batch, narrow / wide: 298 segments
+  // of a median of 3200 keys 112 / 104, 76 of 9700 f64 138 / 136, 32 of 1330 40.4
+  // / 39.2; wide for more, 506 of 86 u64 pairs 50 / 71, 501 of 370 69 / 84)
+  const bool wide = b.num_segments <= 2u * (uint32_t)device_sm_count();
+  cudaError_t e = launch_class<KBITS, PAIRS, 2, false>(b, after_class, s);
+  if (e == cudaSuccess)
+    e = wide ? launch_class<KBITS, PAIRS, 1, true>(b, after_class, s) : launch_class<KBITS, PAIRS, 1, false>(b, after_class, s);
+  if (e == cudaSuccess)
+    e = wide ? launch_class<KBITS, PAIRS, 0, true>(b, after_class, s) : launch_class<KBITS, PAIRS, 0, false>(b, after_class, s);
   return e;
 }
 

@@ -44,8 +44,12 @@
 
 namespace onesweep {
 
+// Not the default at any size: 2^27 u64 pairs take 0.929 ms a pass here and
+// 0.714 in the one-block-per-tile kernel with counting atomics and 5120-key
+// tiles; kept as a variant that a caller or the autotuner may name.
+//
 // Shapes of the persistent kernel: ranker warps, keys per ranker thread and
-// writer warps (measured on GB300 at 2^28 u32 pairs: 24 rankers x 8 keys with
+// writer warps (measured with ballots and lane masks on GB300 at 2^28 u32 pairs: 24 rankers x 8 keys with
 // 8 writers 1.415 ms per pass, 16 x 12 with 8 writers 1.434, with 16 writers
 // 1.462). Shared memory holds one staging buffer and two sorted buffers of a
 // tile, plus the rankers' per-warp digit tables.

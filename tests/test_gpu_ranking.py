@@ -25,7 +25,7 @@ def _dev(a):
     return torch.from_numpy(a.view(np.int64 if a.dtype.itemsize == 8 else np.int32).copy()).cuda()
 
 
-def _check(kt, keys, pairs, begin=0, end=None, descending=False):
+def _check(kt, keys, pairs, begin=0, end=None, descending=False, variant=VARIANT):
     end = KB[kt] if end is None else end
     n = keys.size
     key_type = osw.KEY_TYPES[kt] | (osw.OS_SORT_DESCENDING if descending else 0)
@@ -37,9 +37,9 @@ def _check(kt, keys, pairs, begin=0, end=None, descending=False):
     tail = (n, begin, end, ws.data_ptr(), ws.numel(), s)
     if pairs:
         rc = osw.os_sort_pairs_ex(key_type, k.data_ptr(), ko.data_ptr(), v.data_ptr(), vo.data_ptr(), *tail,
-                                  tile_config=VARIANT)
+                                  tile_config=variant)
     else:
-        rc = osw.os_sort_keys_ex(key_type, k.data_ptr(), ko.data_ptr(), *tail, tile_config=VARIANT)
+        rc = osw.os_sort_keys_ex(key_type, k.data_ptr(), ko.data_ptr(), *tail, tile_config=variant)
     assert rc == osw.OS_OK and osw.os_workspace_status(ws.data_ptr(), s) == osw.OS_OK
     exp = oracle.sort(kt, keys, vals if pairs else None, begin, end, descending=descending)
     ek = exp[0] if pairs else exp
@@ -112,12 +112,13 @@ CLASSES = {32: (4096, 8192, 16384), 64: (2048, 4096, 8192)}
 @pytest.mark.parametrize("kt,pairs,dist,descending", [
     ("u32", True, "uniform", False), ("u32", False, "and5", False), ("u64", True, "and2", True),
     ("f32", True, "normal", True), ("f64", False, "normal", False), ("i32", True, "const", False)])
+@pytest.mark.parametrize("empty", [2, 400])  # few segments: one block of 1024 threads each
 @pytest.mark.parametrize("longest", [0, 1, 60_001])
-def test_batch_class_edges(kt, pairs, dist, descending, longest):
+def test_batch_class_edges(kt, pairs, dist, descending, longest, empty):
     # longest: nothing above the last class, one key above it, or several tiles;
     # with a longer segment, only the first class is sorted in one block
     caps = CLASSES[KB[kt]]
-    sizes = [c + d for c in caps for d in (-1, 0, 1)][:-1] + [0, 1, 33, 256, 257, 1000, 0]
+    sizes = [c + d for c in caps for d in (-1, 0, 1)][:-1] + [0, 1, 33, 256, 257, 1000] + [0] * empty
     sizes += [caps[-1] + longest] if longest else []
     _batch(kt, sizes, pairs, dist, 7, descending)
 
@@ -133,3 +134,13 @@ def test_batch_bit_ranges_of_each_class():
     for begin, end in ((0, 8), (3, 29), (31, 32)):
         _batch("u32", [100, 5000, 9000, 16384, 4096], True, "uniform", 11, begin=begin, end=end)
         _batch("u32", [100, 5000, 9000, 16385, 4096, 40_000], True, "and3", 12, True, begin, end)
+
+
+@pytest.mark.parametrize("kt,pairs", [("u32", True), ("i32", False), ("u64", True), ("f64", False)])
+def test_default_tiles_by_size(kt, pairs):
+    # the default variant at the sizes where its tile changes
+    keys = [osw.os_tile_config_keys(KB[kt], 4 if pairs else 0, VARIANT + g) for g in range(3)]
+    for edge in (152 * 4 * keys[2], 152 * 3 * keys[1], 152 * 3 * keys[0]):
+        for n in (edge, edge + 1):
+            _check(kt, workload.keys(kt, "normal" if kt == "f64" else "and2", n, seed=n), pairs, 0, 13,
+                   variant=None)
