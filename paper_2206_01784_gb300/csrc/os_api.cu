@@ -282,12 +282,12 @@ int make_plan(int key_type, uint64_t n, int value_bytes, int begin_bit, int end_
   }
   // The default variant takes smaller tiles while these make one wave of blocks
   // (geometry 2: 4 an SM, geometry 1: 3): a pass then takes as long as a tile.
-  // us a sort with geometry 0 / 1 / 2, in brackets of 13 key bits: u32 pairs, 1.9M keys 82 / 70 / 68 (52 / 46 / 44), 2.5M 84 /
-  // 73 / 79 (54 / 47 / 48), 3.0M 85 / 99 / 100, 4.2M 121 / 114 / 113, 5.0M 132 /
-  // 124 / 131 (of skewed i32 keys, with cold inputs, 156 / 159), 6.5M 152 / 158 / 163; u32 keys, 1.9M 61 / 55 / 56, 3.0M 65 / 80 /
-  // 82, 5.0M 102 / 93 / 99; u64 pairs, 1.3M 136 / 123 / 126, 2.0M 140 / 175 /
-  // 176, 2.4M 178 / 191 / 191; u64 keys, 1.3M 107 / 100 / 105, 2.4M 145 / 158 /
-  // 160, 3.0M 177 / 169 / 202.
+  // us a sort with geometry 0 / 1 / 2, in brackets of 13 key bits: u32 pairs,
+  // 1.9M keys 82 / 70 / 68 (52 / 46 / 44), 2.5M 84 / 73 / 79 (54 / 47 / 48),
+  // 3.0M 85 / 99 / 100, 5.0M 132 / 124 / 131 (of skewed i32 keys, with cold
+  // inputs, 156 / 159), 6.5M 152 / 158 / 163; u32 keys, 1.9M 61 / 55 / 56, 3.0M
+  // 65 / 80 / 82; u64 pairs, 1.3M 136 / 123 / 126, 2.0M 140 / 175 / 176; u64
+  // keys, 1.3M 107 / 100 / 105, 2.4M 145 / 158 / 160.
   if (set_cfg == kNotSet && radix_bits == kRadixBits) {
     const uint64_t wave1 = 3ull * kSms * tile_keys_for(kb, plan->pairs, kDefaultTileConfig + 1);
     const uint64_t wave2 = 4ull * kSms * tile_keys_for(kb, plan->pairs, kDefaultTileConfig + 2);
