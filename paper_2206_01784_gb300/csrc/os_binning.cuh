@@ -56,6 +56,7 @@
 
 #include "os_common.cuh"
 #include "os_internal.h"
+#include "os_places.h"
 
 namespace onesweep {
 
@@ -414,8 +415,7 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   if (pads) {
     // a ragged tile (the last of its chain) is filled up with keys of the
     // pass's highest digit: they sort behind every key of the tile, are left
-    // out of the published counts, and their places lie past the chain's end,
-    // where the scatter's range check drops them
+    // out of the published counts, and the write-out ends before them
     const K ordered = (K)(mask ^ dxor) << shift;
     const K pad = (FLIP & 1) ? flip_from_ordered(ordered) : ordered;
     for (uint32_t i = c.count + tid; i < (uint32_t)C::T; i += NT) kt[i] = pad;
@@ -566,29 +566,27 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
   K* keys_out = static_cast<K*>(a.keys_out) + c.out_base;
   uint32_t* vals_out = PAIRS ? a.vals_out + c.out_base : nullptr;
   const uint32_t out_len = c.out_len;
+  // (the range check is for a place made from counts that never came: a
+  // look-back that ran past its limit)
   if (homogeneous) {
     const uint32_t g0 = gbase[d0];
-#pragma unroll 4
-    for (int i = 0; i < IPT; ++i) {
-      const uint32_t j = i * NT + tid;
+    for_each_key<NT, kWriteUnroll>(tid, c.count, [&](uint32_t j) {
       const K k = store_transform<FLIP>(load_transform<FLIP>(kt[j]));
       const uint32_t g = g0 + j;
       if (g < out_len) {
         keys_out[g] = k;
         if (PAIRS) vals_out[g] = vt[j];
       }
-    }
+    });
   } else {
-#pragma unroll kWriteUnroll
-    for (int i = 0; i < IPT; ++i) {
-      const uint32_t j = i * NT + tid;
+    for_each_key<NT, kWriteUnroll>(tid, c.count, [&](uint32_t j) {
       const K k = kt[j];
       const uint32_t g = gbase[digit_of(k, shift, mask, dxor)] + j;
       if (g < out_len) {
         keys_out[g] = store_transform<FLIP>(k);
         if (PAIRS) vals_out[g] = vt[j];
       }
-    }
+    });
   }
 }
 
