@@ -125,7 +125,7 @@ OS_API int os_sort_workspace_layout(int key_type, uint64_t n, int value_bytes, i
 /*
  * Sorts of up to about two million keys (12288 32-bit or 8192 64-bit keys per
  * SM of the device) run as one launch that keeps the keys on the chip between
- * passes, unless the caller names a tile variant or a digit width other than 8,
+ * passes, unless the call names a tile variant or a digit width other than 8,
  * the bit range is a single place of more than 4096 keys, or the blocks cannot
  * all be resident at once; the result is the same. On up to 16384 keys the
  * launch is one block or one cluster; above, a cooperative grid.
@@ -290,8 +290,14 @@ OS_API int os_sort_noalloc(int key_type, const void *keys_in, void *keys_out, co
  * are identical under every geometry. Workspaces are sized for the smallest
  * tile, so a workspace sized once fits every geometry. os_set_tile_config
  * returns OS_OK or OS_ERR_INVALID_ARG; os_get_tile_config returns the active
- * geometry or -1.
+ * geometry or -1 for invalid arguments.
+ *
+ * Until a geometry is selected the get calls return OS_TILE_CONFIG_DEFAULT:
+ * variant 4's ranking with the tile chosen by the sort's size. The set calls
+ * take it like any other value, so that setting what was read restores the
+ * state; os_tile_config_keys() gives its largest tile.
  */
+#define OS_TILE_CONFIG_DEFAULT 0x104
 OS_API int os_num_tile_configs(void);
 OS_API int os_tile_config_keys(int key_bits, int value_bytes, int cfg);
 OS_API int os_set_tile_config(int key_bits, int value_bytes, int cfg);
@@ -349,7 +355,8 @@ OS_API int os_profile_stop(os_launch_time *out, int max, int *count);
  * concurrent callers (several host threads, several streams) can each use
  * their own. opt == NULL or opt->tile_config == -1 means the process-wide
  * choice for the sort's size bucket; any other value must be below
- * os_num_tile_configs() (else OS_ERR_INVALID_ARG). Results are identical for
+ * os_num_tile_configs() or OS_TILE_CONFIG_DEFAULT, which is the default
+ * whatever the process-wide choice (else OS_ERR_INVALID_ARG). Results are identical for
  * every variant. The library holds no other per-call state: calls on
  * different streams with different workspaces may run concurrently from any
  * number of host threads.
@@ -358,7 +365,7 @@ OS_API int os_profile_stop(os_launch_time *out, int max, int *count);
  * d = 5..9). 0 means the process-wide choice (os_set_radix_bits_bucket; 8,
  * with 256 bins and p = ceil(bits / 8) passes, until set); 5, 6 or 7 sort
  * with 2^d bins in ceil(bits / d) passes, using tile variant
- * 4 (tile_config must then be -1 or 4) and single arrays only
+ * 4 (tile_config must then be -1, 4 or OS_TILE_CONFIG_DEFAULT) and single arrays only
  * (os_sort_batch_ex rejects them). Any other value: OS_ERR_INVALID_ARG. The
  * sorted output is the same for every d; only the number and cost of the
  * passes change. Workspace sizes do not depend on d.

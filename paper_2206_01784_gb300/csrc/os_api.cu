@@ -86,8 +86,12 @@ constexpr int kTileConfigs = 3 * kGeometries;
 constexpr int kDefaultTileConfig = kGeometries + 0;
 constexpr int kSms = 152;  // of a GB300 (the lines between tile geometries; nothing else depends on it)
 constexpr int kSizeBuckets = 4;  // n < 2^16, < 2^20, < 2^24, larger
-constexpr int kNotSet = -1;  // the default variant, its tile by size
-#define OS_FOUR_DEFAULTS {kNotSet, kNotSet, kNotSet, kNotSet}
+// what the table holds until a variant is set: the default one, its tile by
+// size. A value of its own that callers read and write like any other, so that
+// putting back what was read changes nothing.
+constexpr int kBySize = OS_TILE_CONFIG_DEFAULT;
+static_assert((kBySize & 0xFF) == kDefaultTileConfig && kBySize >= kTileConfigs, "names no variant by itself");
+#define OS_FOUR_DEFAULTS {kBySize, kBySize, kBySize, kBySize}
 int g_tile_cfg[2][2][kSizeBuckets] = {{OS_FOUR_DEFAULTS, OS_FOUR_DEFAULTS}, {OS_FOUR_DEFAULTS, OS_FOUR_DEFAULTS}};
 #undef OS_FOUR_DEFAULTS
 
@@ -101,12 +105,9 @@ int get_radix_bits(int key_bits, bool pairs, int bucket) {
   return v == 0 ? kRadixBits : v;
 }
 
-int raw_tile_cfg(int key_bits, bool pairs, int bucket) {
-  return __atomic_load_n(&g_tile_cfg[key_bits == 64][pairs][bucket], __ATOMIC_RELAXED);
-}
+bool known_tile_cfg(int cfg) { return (cfg >= 0 && cfg < kTileConfigs) || cfg == kBySize; }
 int get_tile_cfg(int key_bits, bool pairs, int bucket) {
-  const int cfg = raw_tile_cfg(key_bits, pairs, bucket);
-  return cfg == kNotSet ? kDefaultTileConfig : cfg;
+  return __atomic_load_n(&g_tile_cfg[key_bits == 64][pairs][bucket], __ATOMIC_RELAXED);
 }
 void set_tile_cfg(int key_bits, bool pairs, int bucket, int cfg) {
   __atomic_store_n(&g_tile_cfg[key_bits == 64][pairs][bucket], cfg, __ATOMIC_RELAXED);
@@ -117,8 +118,6 @@ uint32_t tile_keys_for(int key_bits, bool pairs, int cfg) {
   if (key_bits == 32) return pairs ? binning_tile_keys32_pairs(geo) : binning_tile_keys32_keys(geo);
   return pairs ? binning_tile_keys64_pairs(geo) : binning_tile_keys64_keys(geo);
 }
-
-int binning_config(int key_bits, bool pairs, int bucket) { return get_tile_cfg(key_bits, pairs, bucket); }
 
 // Smallest tile over all geometries: workspaces are sized for it, so any
 // geometry fits a workspace sized once.
@@ -251,7 +250,8 @@ struct Plan {
   os_workspace_layout layout{};
 };
 
-// cfg_override: the caller's binning variant, or -1 for the process-wide one.
+// cfg_override: the caller's binning variant (kBySize: the default), or -1 for
+// the process-wide one.
 // radix_bits: bits per digit place (5-8; narrower digits use tile variant 4,
 // geometry 0 with adaptive ranking), or 0 for the process-wide one (8 when
 // the caller names another variant).
@@ -264,21 +264,19 @@ int make_plan(int key_type, uint64_t n, int value_bytes, int begin_bit, int end_
   if (n >= kMaxKeys) return OS_ERR_TOO_LARGE;
   plan->key_bits = kb;
   plan->pairs = value_bytes == 4;
-  if (radix_bits == 0) {
-    radix_bits = get_radix_bits(kb, plan->pairs, size_bucket(n));
-    if (cfg_override >= 0 && cfg_override != kGeometries) radix_bits = kRadixBits;
-  }
+  if (cfg_override >= 0 && !known_tile_cfg(cfg_override)) return OS_ERR_INVALID_ARG;
+  const bool narrow_ok = cfg_override < 0 || cfg_override == kBySize || cfg_override == kDefaultTileConfig;
+  if (radix_bits == 0) radix_bits = narrow_ok ? get_radix_bits(kb, plan->pairs, size_bucket(n)) : kRadixBits;
   if (radix_bits < kMinRadixBits || radix_bits > kRadixBits) return OS_ERR_INVALID_ARG;
   plan->radix_bits = radix_bits;
   plan->places = (end_bit - begin_bit + radix_bits - 1) / radix_bits;
   plan->bucket = size_bucket(n);
   // the variant is read once: every launch of this sort uses the same one
-  if (cfg_override >= kTileConfigs) return OS_ERR_INVALID_ARG;
-  const int set_cfg = cfg_override >= 0 ? cfg_override : raw_tile_cfg(kb, plan->pairs, plan->bucket);
-  plan->cfg = set_cfg == kNotSet ? kDefaultTileConfig : set_cfg;
+  const int set_cfg = cfg_override >= 0 ? cfg_override : get_tile_cfg(kb, plan->pairs, plan->bucket);
+  plan->cfg = set_cfg == kBySize ? kDefaultTileConfig : set_cfg;
   if (radix_bits != kRadixBits) {
-    if (cfg_override >= 0 && cfg_override != kGeometries) return OS_ERR_INVALID_ARG;
-    plan->cfg = kGeometries;  // geometry 0, adaptive ranking
+    if (!narrow_ok) return OS_ERR_INVALID_ARG;
+    plan->cfg = kDefaultTileConfig;  // geometry 0, adaptive ranking
   }
   // The default variant takes smaller tiles while these make one wave of blocks
   // (geometry 2: 4 an SM, geometry 1: 3): a pass then takes as long as a tile.
@@ -288,7 +286,7 @@ int make_plan(int key_type, uint64_t n, int value_bytes, int begin_bit, int end_
   // inputs, 156 / 159), 6.5M 152 / 158 / 163; u32 keys, 1.9M 61 / 55 / 56, 3.0M
   // 65 / 80 / 82; u64 pairs, 1.3M 136 / 123 / 126, 2.0M 140 / 175 / 176; u64
   // keys, 1.3M 107 / 100 / 105, 2.4M 145 / 158 / 160.
-  if (set_cfg == kNotSet && radix_bits == kRadixBits) {
+  if (set_cfg == kBySize && radix_bits == kRadixBits) {
     const uint64_t wave1 = 3ull * kSms * tile_keys_for(kb, plan->pairs, kDefaultTileConfig + 1);
     const uint64_t wave2 = 4ull * kSms * tile_keys_for(kb, plan->pairs, kDefaultTileConfig + 2);
     if (n <= wave2)
@@ -498,7 +496,8 @@ int run_sort(int key_type, const void* keys_in, void* keys_out, const uint32_t* 
     return OS_OK;
   }
 
-  if (cfg_override < 0 && run_small(plan, key_type, keys_in, keys_out, vals_in, vals_out, n, begin_bit, end_bit, w, s, &rc))
+  if ((cfg_override < 0 || cfg_override == kBySize) &&
+      run_small(plan, key_type, keys_in, keys_out, vals_in, vals_out, n, begin_bit, end_bit, w, s, &rc))
     return rc;
 
   // zero: status word, done counter, histograms, this sort's tile counters
@@ -629,8 +628,9 @@ int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int va
   bp->pairs = value_bytes == 4;
   bp->places = (end_bit - begin_bit + kRadixBits - 1) / kRadixBits;
   bp->bucket = size_bucket(S > 0 ? n_total / S : n_total);  // by the mean segment length
-  if (cfg_override >= kTileConfigs) return OS_ERR_INVALID_ARG;
-  bp->cfg = cfg_override >= 0 ? cfg_override : binning_config(kb, bp->pairs, bp->bucket);
+  if (cfg_override >= 0 && !known_tile_cfg(cfg_override)) return OS_ERR_INVALID_ARG;
+  const int set_cfg = cfg_override >= 0 ? cfg_override : get_tile_cfg(kb, bp->pairs, bp->bucket);
+  bp->cfg = set_cfg == kBySize ? kDefaultTileConfig : set_cfg;
   bp->fault_tile = g_fault_tile.load(std::memory_order_relaxed);
   bp->spin_limit = g_spin_limit.load(std::memory_order_relaxed);
   // the default variant takes smaller tiles while the batch is small: with
@@ -639,7 +639,7 @@ int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int va
   // / 2: 298 segments, 1.8M f32 pairs 125 / 110 / 107; 232, 3.1M f32 pairs 168 /
   // 148 / 143; 256, 8.8M i32 keys 220 / 232 / 232; 16, 0.1M f64 keys 111 / 103 /
   // 92; 76, 1.6M f64 pairs 185 / 173 / 194)
-  if (cfg_override < 0 && bp->cfg == kDefaultTileConfig) {
+  if ((cfg_override < 0 || cfg_override == kBySize) && bp->cfg == kDefaultTileConfig) {
     const uint64_t wave = kb == 32 ? 4u << 20 : 5u << 18;
     if (n_total <= wave)
       bp->cfg += 2;
@@ -898,7 +898,7 @@ static int option_config(const os_sort_options* opt, int* cfg, int* radix_bits) 
   *cfg = -1;
   *radix_bits = 0;
   if (!opt) return OS_OK;
-  if (opt->tile_config < -1 || opt->tile_config >= kTileConfigs) return OS_ERR_INVALID_ARG;
+  if (opt->tile_config != -1 && !known_tile_cfg(opt->tile_config)) return OS_ERR_INVALID_ARG;
   if (opt->radix_bits != 0 && (opt->radix_bits < (uint32_t)kMinRadixBits || opt->radix_bits > (uint32_t)kRadixBits))
     return OS_ERR_INVALID_ARG;
   *cfg = opt->tile_config;
@@ -1046,15 +1046,15 @@ const char* os_build_info(void) { return "cuda_arch_list=" OS_STR(__CUDA_ARCH_LI
 int os_num_tile_configs(void) { return kTileConfigs; }
 
 int os_tile_config_keys(int key_bits, int value_bytes, int cfg) {
-  if ((key_bits != 32 && key_bits != 64) || (value_bytes != 0 && value_bytes != 4) || cfg < 0 ||
-      cfg >= kTileConfigs)
+  if ((key_bits != 32 && key_bits != 64) || (value_bytes != 0 && value_bytes != 4) ||
+      !known_tile_cfg(cfg))
     return 0;
   return (int)tile_keys_for(key_bits, value_bytes == 4, cfg);
 }
 
 int os_set_tile_config(int key_bits, int value_bytes, int cfg) {
-  if ((key_bits != 32 && key_bits != 64) || (value_bytes != 0 && value_bytes != 4) || cfg < 0 ||
-      cfg >= kTileConfigs)
+  if ((key_bits != 32 && key_bits != 64) || (value_bytes != 0 && value_bytes != 4) ||
+      !known_tile_cfg(cfg))
     return OS_ERR_INVALID_ARG;
   for (int b = 0; b < kSizeBuckets; ++b) set_tile_cfg(key_bits, value_bytes == 4, b, cfg);
   return OS_OK;
@@ -1070,8 +1070,8 @@ int os_num_size_buckets(void) { return kSizeBuckets; }
 int os_size_bucket(uint64_t n) { return size_bucket(n); }
 
 int os_set_tile_config_bucket(int key_bits, int value_bytes, int bucket, int cfg) {
-  if ((key_bits != 32 && key_bits != 64) || (value_bytes != 0 && value_bytes != 4) || cfg < 0 ||
-      cfg >= kTileConfigs || bucket < 0 || bucket >= kSizeBuckets)
+  if ((key_bits != 32 && key_bits != 64) || (value_bytes != 0 && value_bytes != 4) ||
+      !known_tile_cfg(cfg) || bucket < 0 || bucket >= kSizeBuckets)
     return OS_ERR_INVALID_ARG;
   set_tile_cfg(key_bits, value_bytes == 4, bucket, cfg);
   return OS_OK;

@@ -174,9 +174,7 @@ cudaError_t launch_batch_class_sorts(int key_bits, bool pairs, const BatchArgs& 
 cudaError_t launch_batch_histogram(int key_bits, const BatchArgs& b, bool after_class, cudaStream_t s);
 uint32_t batch_class_capacity(int key_bits, int cls);
 
-// Active binning variant for a key width / payload / size bucket, and the
-// tile size of a variant.
-int binning_config(int key_bits, bool pairs, int bucket);
+// Keys per tile of a binning variant.
 uint32_t tile_keys_for(int key_bits, bool pairs, int cfg);
 
 int sort_on_workspace(int key_type, const void* keys_in, void* keys_out, const uint32_t* vals_in, uint32_t* vals_out,

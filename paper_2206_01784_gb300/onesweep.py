@@ -23,6 +23,7 @@ KEY_BITS = {OS_KEY_U32: 32, OS_KEY_U64: 64, OS_KEY_F32: 32, OS_KEY_F64: 64, OS_K
 
 OS_OK, OS_ERR_INVALID_ARG, OS_ERR_TOO_LARGE, OS_ERR_WORKSPACE, OS_ERR_CUDA, OS_ERR_TIMEOUT = range(6)
 OS_ERR_SCRATCH_LIMIT = 6
+OS_TILE_CONFIG_DEFAULT = 0x104  # adaptive ranking, the tile by the sort's size (until a variant is set)
 OS_HOST_COPY_ENGINES, OS_HOST_COPY_LINK = 0, 1  # how the host-memory sorts move data
 
 

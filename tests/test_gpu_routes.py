@@ -1,0 +1,147 @@
+"""Sorts by the route they take, bit-exact against the oracle.
+
+A sort that names a tile variant runs pass by pass whatever its size, so the
+variants' kernels are reached by naming them, with both payloads; the sizes of
+the cluster form are those around its 8 and 16 blocks; and the default's tile
+is asserted beside the sorts that rely on it.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+from paper_2206_01784_gb300 import autotune  # noqa: E402
+from paper_2206_01784_gb300 import onesweep as osw  # noqa: E402
+from paper_2206_01784_gb300 import workload  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+KB = {"u32": 32, "u64": 64, "f32": 32, "f64": 64, "i32": 32, "i64": 64}
+DEFAULT = osw.OS_TILE_CONFIG_DEFAULT
+
+
+def _dev(a, shift=0):
+    """A copy on the device, `shift` elements past an aligned address."""
+    t = torch.from_numpy(np.concatenate([np.zeros(shift, a.dtype), a]).view(np.int64 if a.dtype.itemsize == 8 else np.int32))
+    return t.cuda()[shift:]
+
+
+def _check(kt, keys, pairs, variant=None, begin=0, end=None, descending=False, shift=0, radix_bits=None):
+    end = KB[kt] if end is None else end
+    n = keys.size
+    key_type = osw.KEY_TYPES[kt] | (osw.OS_SORT_DESCENDING if descending else 0)
+    vals = workload.iota_u32(n)
+    k, v = _dev(keys, shift), _dev(vals, shift)
+    ko, vo = _dev(np.zeros_like(keys), shift), _dev(np.zeros_like(vals), shift)
+    ws = osw.workspace(key_type, n, 4 if pairs else 0, begin, end, k.device).random_(0, 256)
+    s = torch.cuda.current_stream().cuda_stream
+    tail = (n, begin, end, ws.data_ptr(), ws.numel(), s)
+    opts = dict(tile_config=variant, radix_bits=radix_bits)
+    if pairs:
+        rc = osw.os_sort_pairs_ex(key_type, k.data_ptr(), ko.data_ptr(), v.data_ptr(), vo.data_ptr(), *tail, **opts)
+    else:
+        rc = osw.os_sort_keys_ex(key_type, k.data_ptr(), ko.data_ptr(), *tail, **opts)
+    assert rc == osw.OS_OK and osw.os_workspace_status(ws.data_ptr(), s) == osw.OS_OK
+    exp = oracle.sort(kt, keys, vals if pairs else None, begin, end, descending=descending)
+    ek = exp[0] if pairs else exp
+    assert np.array_equal(ko.cpu().numpy().view(ek.dtype), ek)
+    assert not pairs or np.array_equal(vo.cpu().numpy().view(np.uint32), exp[1])
+
+
+def _keys(kt, dist, n, seed):
+    return workload.keys(kt, "normal" if kt[0] == "f" else dist, n, seed=seed)
+
+
+@pytest.mark.parametrize("pairs", [True, False])
+@pytest.mark.parametrize("kt", ["u32", "u64", "f32", "i64"])
+@pytest.mark.parametrize("cfg", range(12))
+def test_every_variant_with_both_payloads(cfg, kt, pairs):
+    t = osw.os_tile_config_keys(KB[kt], 4 if pairs else 0, cfg)
+    for n in (t - 1, 2 * t, 5 * t + 3):
+        _check(kt, _keys(kt, "and2", n, cfg * 7 + n), pairs, cfg)
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+@pytest.mark.parametrize("kt,pairs,cfg", [("u32", True, 4), ("u32", False, 4), ("u64", True, 4), ("u64", False, 6),
+                                          ("f32", True, 5), ("u32", True, 7), ("u64", True, 7), ("f64", False, 3)])
+def test_pass_by_pass_at_any_address(kt, pairs, cfg, shift):
+    t = osw.os_tile_config_keys(KB[kt], 4 if pairs else 0, cfg)
+    for n in (t + 1, 7 * t - 5):
+        _check(kt, _keys(kt, "and2", n, n), pairs, cfg, shift=shift)
+
+
+@pytest.mark.parametrize("seed", range(16))
+def test_random_sorts_pass_by_pass(seed):
+    rng = np.random.default_rng(1000 + seed)
+    kt = str(rng.choice(list(KB)))
+    n = int(np.exp(rng.uniform(np.log(1), np.log(400_000))))
+    begin = int(rng.integers(0, KB[kt] - 1)) if kt[0] != "f" and rng.random() < 0.5 else 0
+    end = int(rng.integers(begin + 1, KB[kt] + 1)) if kt[0] != "f" and rng.random() < 0.5 else KB[kt]
+    dist = str(rng.choice(["uniform", "and2", "and3", "and8", "const"]))
+    _check(kt, _keys(kt, dist, n, seed), bool(rng.integers(2)), int(rng.integers(12)), begin, end,
+           bool(rng.integers(2)), int(rng.integers(4)))
+
+
+CLUSTERS = [4097, 6000, 8191, 8192, 8193, 9 * 1024, 9 * 1024 + 1, 15 * 1024 + 1, 16383, 16384, 16385]
+
+
+@pytest.mark.parametrize("n", CLUSTERS)
+@pytest.mark.parametrize("kt,dist,begin,end,descending", [
+    ("u32", "uniform", 0, 32, False), ("f32", "normal", 0, 32, True), ("i64", "and3", 7, 64, True),
+    ("f64", "normal", 0, 64, False), ("u64", "const", 0, 40, False), ("i32", "and8", 0, 31, False)])
+def test_clusters(n, kt, dist, begin, end, descending):
+    for pairs in (True, False):
+        _check(kt, _keys(kt, dist, n, n), pairs, None, begin, end, descending, shift=n % 4)
+
+
+def test_clusters_on_several_streams_and_in_a_graph():
+    sizes = (6000, 9217, 16384, 12_345, 16384, 5000)
+    work = []
+    for i, n in enumerate(sizes):
+        keys = _keys("u32", "and2", n, i)
+        work.append((keys, _dev(keys), _dev(workload.iota_u32(n)), torch.cuda.Stream(),
+                     osw.workspace(osw.OS_KEY_U32, n, 4, 0, 32, "cuda")))
+    torch.cuda.synchronize()
+    # (outputs of every round are kept: the allocator knows nothing of the streams)
+    outs = [[osw.sort_pairs(k, v, key_type="u32", ws=ws, stream=s) for _, k, v, s, ws in work] for _ in range(4)]
+    torch.cuda.synchronize()
+    for (keys, *_), (ko, vo) in zip(work * len(outs), sum(outs, [])):
+        ek, ev = oracle.sort("u32", keys, workload.iota_u32(keys.size))
+        assert np.array_equal(ko.cpu().numpy().view(np.uint32), ek) and np.array_equal(vo.cpu().numpy().view(np.uint32), ev)
+    for _, k, v, _, ws in work:
+        ko, vo = torch.empty_like(k), torch.empty_like(v)
+        run = lambda: osw.sort_pairs(k, v, key_type="u32", keys_out=ko, values_out=vo, ws=ws)  # noqa: E731
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            run()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            run()
+        keys = _keys("u32", "and3", k.numel(), 77)
+        k.copy_(_dev(keys))
+        ws.random_(0, 256)
+        graph.replay()
+        torch.cuda.synchronize()
+        ek, ev = oracle.sort("u32", keys, workload.iota_u32(keys.size))
+        assert np.array_equal(ko.cpu().numpy().view(np.uint32), ek) and np.array_equal(vo.cpu().numpy().view(np.uint32), ev)
+
+
+@pytest.mark.parametrize("kt,pairs", [("u32", True), ("u64", False)])
+def test_default_by_size_is_what_runs(kt, pairs):
+    vb, saved = 4 if pairs else 0, autotune.current()
+    tiles = [osw.os_tile_config_keys(KB[kt], vb, 4 + g) for g in range(3)]
+    try:
+        for variant in (None, DEFAULT):
+            # (named for the call, the default holds whatever the process-wide variant)
+            assert osw.os_set_tile_config(KB[kt], vb, DEFAULT if variant is None else 0) == osw.OS_OK
+            for edge, below, above in ((152 * 4 * tiles[2], tiles[2], tiles[1]), (152 * 3 * tiles[1], tiles[1], tiles[0])):
+                for n, tile in ((edge, below), (edge + 1, above)):
+                    if variant is None:
+                        assert osw.os_sort_workspace_layout(osw.KEY_TYPES[kt], n, vb, 0, 13).tile_keys == tile
+                    _check(kt, _keys(kt, "and2", n, n % 97), pairs, variant, 0, 13)
+        _check(kt, _keys(kt, "and2", 100_003, 3), pairs, DEFAULT, radix_bits=6)
+    finally:
+        autotune.apply(saved)
+
