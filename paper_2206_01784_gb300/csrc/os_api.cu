@@ -639,11 +639,10 @@ int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int va
   // / 2: 298 segments, 1.8M f32 pairs 125 / 110 / 107; 232, 3.1M f32 pairs 168 /
   // 148 / 143; 256, 8.8M i32 keys 220 / 232 / 232; 16, 0.1M f64 keys 111 / 103 /
   // 92; 76, 1.6M f64 pairs 185 / 173 / 194)
-  if ((cfg_override < 0 || cfg_override == kBySize) && bp->cfg == kDefaultTileConfig) {
-    const uint64_t wave = kb == 32 ? 4u << 20 : 5u << 18;
-    if (n_total <= wave)
+  if (set_cfg == kBySize) {
+    if (n_total <= (kb == 32 ? 4u << 20 : 5u << 18))
       bp->cfg += 2;
-    else if (n_total <= (kb == 32 ? wave : 2 * wave))
+    else if (kb == 64 && n_total <= 5u << 19)
       bp->cfg += 1;
   }
   // the persistent kernel serves single arrays: a batch runs geometry 0 with
@@ -651,7 +650,7 @@ int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int va
   if (bp->cfg % kGeometries == kPersistentGeometry) bp->cfg -= kPersistentGeometry;
   bp->tile = tile_keys_for(kb, bp->pairs, bp->cfg);
   const uint32_t min_tile = min_tile_keys(kb, bp->pairs);
-  // (n_total keys that fit class 1 make no large segment)
+  // (n_total keys that fit the last class make no large segment)
   bp->max_large = n_total > batch_class_capacity(kb, kBatchClasses - 1) ? n_total / (batch_class_capacity(kb, 0) + 1) : 0;
   if (bp->max_large > S) bp->max_large = S;
   bp->max_tiles = n_total / min_tile + bp->max_large;

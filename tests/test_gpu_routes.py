@@ -145,3 +145,29 @@ def test_default_by_size_is_what_runs(kt, pairs):
     finally:
         autotune.apply(saved)
 
+
+
+@pytest.mark.parametrize("cfg", [4, 5, 6, DEFAULT])
+@pytest.mark.parametrize("by_call", [True, False])
+def test_a_batch_runs_the_variant_that_was_set(cfg, by_call):
+    # word 2 of the workspace: the tiles that the plan laid out
+    sizes = [100_000, 50_001, 70_000]
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    keys, vals, n = _keys("u32", "and2", int(offs[-1]), 5), workload.iota_u32(int(offs[-1])), int(offs[-1])
+    tile = osw.os_tile_config_keys(32, 4, 6 if cfg == DEFAULT else cfg)  # (by size: a small batch, small tiles)
+    k, v, o = _dev(keys), _dev(vals), torch.from_numpy(offs).cuda()
+    ko, vo = torch.empty_like(k), torch.empty_like(v)
+    ws = osw.batch_workspace(osw.OS_KEY_U32, n, len(sizes), 4, 0, 32, "cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    saved = autotune.current()
+    try:
+        assert osw.os_set_tile_config(32, 4, 0 if by_call else cfg) == osw.OS_OK
+        assert osw.os_sort_batch_ex(osw.OS_KEY_U32, k.data_ptr(), ko.data_ptr(), v.data_ptr(), vo.data_ptr(),
+                                    o.data_ptr(), len(sizes), n, 0, 32, ws.data_ptr(), ws.numel(), s,
+                                    tile_config=cfg if by_call else None) == osw.OS_OK
+        assert osw.os_workspace_status(ws.data_ptr(), s) == osw.OS_OK
+    finally:
+        autotune.apply(saved)
+    assert int(ws[8:12].cpu().numpy().view(np.uint32)[0]) == sum((x + tile - 1) // tile for x in sizes)
+    ek, ev = oracle.sort_segments("u32", keys, offs.astype(np.uint64), vals)
+    assert np.array_equal(ko.cpu().numpy().view(np.uint32), ek) and np.array_equal(vo.cpu().numpy().view(np.uint32), ev)
