@@ -7,7 +7,9 @@ bits make each pass cheaper and the sort longer), and keeps one active
 (variant, d) per (key width, payload, size bucket). ``tune`` times every
 variant at d = 8 and variant 4 (the one narrower digits run) at each smaller
 d on seeded uniform keys of a size representative of each bucket (CUDA events
-around whole sorts), installs the fastest through os_set_tile_config_bucket
+around whole sorts), beside the default (one launch for the sorts that fit
+it, the tile by size for the others), which a named variant has to beat by
+more than MARGIN; installs the fastest through os_set_tile_config_bucket
 and os_set_radix_bits_bucket and returns the table; ``save`` / ``load`` /
 ``apply`` keep tables across processes. Results of a sort never depend on the
 variant or on d - only its speed does - and workspaces are sized for the
@@ -28,6 +30,7 @@ BUCKET_SIZES = {0: 1 << 15, 1: 1 << 19, 2: 1 << 23, 3: 1 << 26}
 
 NARROW_VARIANT = 4          # the tile variant of digits narrower than 8 bits
 RADIX_BITS = (5, 6, 7, 8)  # digit widths the library carries
+MARGIN = 0.03               # the default follows the size within a bucket; a tie with it is noise
 
 
 def _time_sort(kt, k, v, ko, vo, n, kb, ws, steps, warmup, torch, cfg=None, radix_bits=None):
@@ -65,10 +68,12 @@ def candidates(radix_bits=RADIX_BITS):
 
 def tune(key_bits=(32, 64), value_bytes=(0, 4), buckets=None, steps: int = 5, warmup: int = 2, seed: int = 1234,
          sizes: dict | None = None, verbose: bool = False, radix_bits=RADIX_BITS) -> dict:
-    """Times every candidate and installs the fastest per (key bits, value bytes, bucket).
+    """Times every candidate and installs the fastest per (key bits, value bytes, bucket),
+    or the default (osw.OS_TILE_CONFIG_DEFAULT) where no candidate beats it.
 
     Returns {(key_bits, value_bytes, bucket): {"cfg": variant, "radix_bits": d,
-    "ms": {"cfg/d": ms}, "n": keys}}."""
+    "ms": {"cfg/d": ms}, "default_ms": ms, "n": keys}} (without default_ms where
+    radix_bits leaves out 8)."""
     import numpy as np
     import torch
 
@@ -93,13 +98,21 @@ def tune(key_bits=(32, 64), value_bytes=(0, 4), buckets=None, steps: int = 5, wa
                 for cfg, d in candidates(radix_bits):
                     times[(cfg, d)] = _time_sort(kt, k, v, ko, vo, n, kb, ws, steps, warmup, torch, cfg, d)
                 best = min(times, key=times.__getitem__)
+                best_ms, default_ms = times[best], None
+                if 8 in radix_bits:
+                    default_ms = _time_sort(kt, k, v, ko, vo, n, kb, ws, steps, warmup, torch,
+                                            osw.OS_TILE_CONFIG_DEFAULT, 8)
+                    if best_ms > (1.0 - MARGIN) * default_ms:
+                        best, best_ms = (osw.OS_TILE_CONFIG_DEFAULT, 8), default_ms
                 osw.os_set_tile_config_bucket(kb, vb, b, best[0])
                 osw.os_set_radix_bits_bucket(kb, vb, b, best[1])
                 table[(kb, vb, b)] = {"cfg": best[0], "radix_bits": best[1],
                                       "ms": {f"{c}/{d}": t for (c, d), t in times.items()}, "n": n}
+                if default_ms is not None:
+                    table[(kb, vb, b)]["default_ms"] = default_ms
                 if verbose:
                     print(f"key_bits={kb} value_bytes={vb} bucket={b} n={n}: variant {best[0]}, {best[1]}-bit "
-                          f"digits ({times[best]:.3f} ms)", flush=True)
+                          f"digits ({best_ms:.3f} ms)", flush=True)
                 del k, ko, v, vo, ws
     return table
 
