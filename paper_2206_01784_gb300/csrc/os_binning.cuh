@@ -469,7 +469,9 @@ __device__ __forceinline__ void binning_tile(const PassArgs& a, unsigned char* s
     if (lane >= o) incl += y;
   }
   if (lane == 31) misc[warp] = incl;
-  if (filled == (uint32_t)C::T) misc[NW] = 1u;
+  // (without the pads: all-equal keys would otherwise rank one tile, the last,
+  // in every pass; 4.0M u32 pairs 95 us a sort so, 70 as it is)
+  if (digit_count == c.count) misc[NW] = 1u;
   __syncthreads();
   const bool homogeneous = misc[NW] != 0u;
 
