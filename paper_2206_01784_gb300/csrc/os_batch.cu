@@ -5,7 +5,8 @@
 //
 //  * plan: one block reads the segment boundaries on the device and lays out
 //    the work. Segments of up to one block's capacity are listed by class for
-//    the one-block sorts; each longer ("large") segment gets a row of its own, consecutive tile ids (its look-back chain) and histogram work items.
+//    the one-block sorts; each longer ("large") segment gets a row of its own,
+//    consecutive tile ids (its look-back chain) and histogram work items.
 //    Nothing is read back to the host, so a batch can be captured in a CUDA
 //    graph;
 //  * one-block sorts: blocks take the listed segments one after another and
@@ -340,13 +341,16 @@ __global__ void __launch_bounds__(ClassTile<KBITS, PAIRS, CLS, WIDE>::kClass.thr
   if (blockIdx.x == 0) pdl_wait();
 }
 
+// Dynamic shared memory of which `blocks` fit an SM (228 KB, of which each
+// block takes 1 KB besides) and one more does not.
+constexpr size_t smem_for_blocks(int blocks) {
+  return (228 * 1024 / (size_t)(blocks + 1) - 1024 + 128) / 128 * 128;
+}
+
 template <int KBITS, bool PAIRS, int CLS, bool WIDE>
 cudaError_t launch_class(const BatchArgs& b, bool* after_kernel, cudaStream_t s) {
   using CT = ClassTile<KBITS, PAIRS, CLS, WIDE>;
   auto* kernel = batch_class_sort_kernel<KBITS, PAIRS, CLS, WIDE>;
-  // set on every launch: an idempotent host-side attribute
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CT::Tile::smem_bytes);
-  if (e != cudaSuccess) return e;
   const int sms = device_sm_count();
   if (sms <= 0) return cudaErrorInvalidConfiguration;
   // at most one block per segment the class can have, by the class below's capacity
@@ -354,7 +358,21 @@ cudaError_t launch_class(const BatchArgs& b, bool* after_kernel, cudaStream_t s)
   if (grid > b.num_segments) grid = b.num_segments;
   if (grid > (uint64_t)sms * CT::kClass.blocks_per_sm) grid = (uint64_t)sms * CT::kClass.blocks_per_sm;
   if (grid == 0) return cudaSuccess;
-  e = launch_kernel(kernel, (unsigned)grid, CT::kClass.threads, CT::Tile::smem_bytes, s, *after_kernel, b);
+  // The kernel starts while blocks of the one before still hold most SMs, and
+  // its own would fill up the few that are free: a grid of fewer blocks than
+  // the device holds takes more shared memory, so that no SM takes more than
+  // its share. us a batch of u32 pairs without and with it: 305 segments of
+  // 4096 keys 55.3 / 48.7, of 3000 49.5 / 43.4 (600 of 4096 63.4 / 63.5: four
+  // blocks an SM either way); u64 pairs, 305 of 1000 51.2 / 47.1.
+  constexpr size_t least = CT::Tile::smem_bytes;
+  constexpr size_t most = smem_for_blocks(1) > least ? smem_for_blocks(1) : least;
+  const int share = (int)((grid + sms - 1) / sms);
+  size_t bytes = share < CT::kClass.blocks_per_sm ? smem_for_blocks(share) : least;
+  if (bytes < least) bytes = least;
+  // set on every launch, and always to the most: an idempotent host-side attribute
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (e != cudaSuccess) return e;
+  e = launch_kernel(kernel, (unsigned)grid, CT::kClass.threads, bytes, s, *after_kernel, b);
   *after_kernel = true;
   return e;
 }
@@ -363,16 +381,23 @@ cudaError_t launch_class(const BatchArgs& b, bool* after_kernel, cudaStream_t s)
 // first of them waits for the plan as any kernel does.
 template <int KBITS, bool PAIRS>
 cudaError_t launch_classes(const BatchArgs& b, bool* after_class, cudaStream_t s) {
-  // few segments: every SM has one or two, whose own time counts, so a segment
-  // gets a whole block of 1024 threads (us a batch, narrow / wide: 298 segments
-  // of a median of 3200 keys 112 / 104, 76 of 9700 f64 138 / 136, 32 of 1330 40.4
-  // / 39.2; wide for more, 506 of 86 u64 pairs 50 / 71, 501 of 370 69 / 84)
-  const bool wide = b.num_segments <= 2u * (uint32_t)device_sm_count();
+  // At most one segment an SM, and more keys than half of class 0's capacity on
+  // the mean: a segment's own time counts, so it gets a whole block of 1024
+  // threads. us a batch of u32 pairs, blocks of 256 or 512 / 1024: 16 segments
+  // of 4096 keys 30.7 / 28.7, of 8000 36.9 / 34.9 (AND of 3 words 43.0 / 34.8,
+  // 49.2 / 45.1); shorter ones leave most of the threads idle: 152 of 1000 24.6
+  // / 28.5, of 20 16.4 / 18.4; so do 64-bit keys: 152 of 4096 54.5 / 57.4, 16
+  // 47.1 / 47.1. Two segments an SM take turns: 304 of 4096 45.1 / 50.7, of 86
+  // 28.6 / 32.8, 304 of 1000 u64 45.0 / 56.9.
+  const bool wide = KBITS == 32 && b.num_segments <= (uint32_t)device_sm_count() &&
+                    b.n_total >= (uint64_t)b.num_segments * (b.class_max[0] / 2);
   cudaError_t e = launch_class<KBITS, PAIRS, 2, false>(b, after_class, s);
-  if (e == cudaSuccess)
-    e = wide ? launch_class<KBITS, PAIRS, 1, true>(b, after_class, s) : launch_class<KBITS, PAIRS, 1, false>(b, after_class, s);
-  if (e == cudaSuccess)
-    e = wide ? launch_class<KBITS, PAIRS, 0, true>(b, after_class, s) : launch_class<KBITS, PAIRS, 0, false>(b, after_class, s);
+  if constexpr (KBITS == 32) {
+    if (e == cudaSuccess && wide) e = launch_class<KBITS, PAIRS, 1, true>(b, after_class, s);
+    if (e == cudaSuccess && wide) e = launch_class<KBITS, PAIRS, 0, true>(b, after_class, s);
+  }
+  if (e == cudaSuccess && !wide) e = launch_class<KBITS, PAIRS, 1, false>(b, after_class, s);
+  if (e == cudaSuccess && !wide) e = launch_class<KBITS, PAIRS, 0, false>(b, after_class, s);
   return e;
 }
 

@@ -171,3 +171,21 @@ def test_a_batch_runs_the_variant_that_was_set(cfg, by_call):
     assert int(ws[8:12].cpu().numpy().view(np.uint32)[0]) == sum((x + tile - 1) // tile for x in sizes)
     ek, ev = oracle.sort_segments("u32", keys, offs.astype(np.uint64), vals)
     assert np.array_equal(ko.cpu().numpy().view(np.uint32), ek) and np.array_equal(vo.cpu().numpy().view(np.uint32), ev)
+
+
+@pytest.mark.parametrize("segments", [1, 100, 152, 153, 304, 305, 457, 700])
+@pytest.mark.parametrize("kt,pairs,dist", [("u32", True, "and2"), ("u64", True, "uniform"), ("f32", False, "normal")])
+def test_batches_by_blocks_an_sm(segments, kt, pairs, dist):
+    # one to four blocks an SM, of 256 threads or (few long segments) of 1024
+    cap = 4096 if KB[kt] == 32 else 2048
+    for lo, hi in ((1, 200), (cap // 2, cap), (cap // 2, 4 * cap)):
+        sizes = np.random.default_rng(segments).integers(lo, hi + 1, segments)
+        offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        keys, vals = _keys(kt, dist, int(offs[-1]), segments), workload.iota_u32(int(offs[-1]))
+        ws = osw.batch_workspace(osw.KEY_TYPES[kt], keys.size, segments, 4 if pairs else 0, 0, KB[kt], "cuda").random_(0, 256)
+        out = osw.sort_batch(_dev(keys), torch.from_numpy(offs).cuda(), _dev(vals) if pairs else None, key_type=kt, ws=ws)
+        assert osw.os_workspace_status(ws.data_ptr(), torch.cuda.current_stream().cuda_stream) == osw.OS_OK
+        exp = oracle.sort_segments(kt, keys, offs.astype(np.uint64), vals if pairs else None)
+        ko, ek = (out[0], exp[0]) if pairs else (out, exp)
+        assert np.array_equal(ko.cpu().numpy().view(ek.dtype), ek)
+        assert not pairs or np.array_equal(out[1].cpu().numpy().view(np.uint32), exp[1])
