@@ -9,8 +9,9 @@ namespace onesweep {
 
 // SPREAD: the tile's keys are spread evenly over the block's threads (ceil(n /
 // NT) each) rather than filling the first warps with IPT a thread, so that a
-// tile takes time by its length; for tiles that are whole sorts. APART: a digit
-// that many keys of a warp share is ranked apart.
+// tile takes time by its length; for tiles that are whole sorts. APART (whole
+// sorts of keys of any kind): a digit that many keys of a warp share is ranked
+// apart, and places that all keys share are passed over.
 template <int KBITS, bool PAIRS, int NT_, int IPT_, bool SPREAD = false, bool APART = false>
 struct SmallTile {
   using K = typename KeyWord<KBITS>::type;
@@ -29,7 +30,8 @@ struct SmallTile {
   static constexpr size_t wcnt = vbuf + (PAIRS ? (size_t)T * 4 : 0);  // [NW][256] running counts of each warp
   static constexpr size_t psum = wcnt + (size_t)NW * kRadix * 4;      // [Q][256] digit counts of a part
   static constexpr size_t gsum = psum + (size_t)Q * kRadix * 4;       // [Q][8] ... of 32 digits
-  static constexpr size_t smem_bytes = gsum + 32 * 4;
+  static constexpr size_t dsum = gsum + 32 * 4;  // APART: [NW] bits that differ in a warp, [NW] its first key
+  static constexpr size_t smem_bytes = dsum + (APART ? 2 * NW * sizeof(K) : 0);
 
   K key[IPT];
   uint32_t val[PAIRS ? IPT : 1];
@@ -62,7 +64,8 @@ struct SmallTile {
   template <bool kL2 = false>
   __device__ __forceinline__ void load_keys(const K* keys, int flip = 0) {
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) key[i] = !valid(i) ? K(0) : kL2 ? __ldcg(keys + wbase + i * 32) : keys[wbase + i * 32];
+    for (int i = 0; i < IPT; ++i)
+      key[i] = !valid(i) ? K(0) : kL2 ? __ldcg(keys + wbase + i * 32) : keys[wbase + i * 32];
     if (flip) {
 #pragma unroll
       for (int i = 0; i < IPT; ++i) key[i] = flip_to_ordered(key[i]);
@@ -87,9 +90,11 @@ struct SmallTile {
   // and that of the shared-memory round trips between them. So the scan over
   // 256 digits takes no barrier of its own: each warp adds the sums of the
   // lower groups of 32 digits itself (one load, one warp reduction).
+  // note (APART): each warp leaves the bits in which its keys differ, for
+  // differing_bits().
   template <typename Values, typename Publish>
   __device__ __forceinline__ void bin(unsigned char* smem, int shift, uint32_t mask, uint32_t dxor, Values values,
-                                      Publish publish) {
+                                      Publish publish, bool note = false) {
     constexpr int U = IPT % 4 == 0 ? 4 : 2;
     K* kb = reinterpret_cast<K*>(smem + kbuf);
     uint32_t* vb = reinterpret_cast<uint32_t*>(smem + vbuf);
@@ -104,10 +109,45 @@ struct SmallTile {
     // keys share (the most frequent of four sampled lanes') is ranked by votes,
     // for its atomics would all meet in one counter
     uint32_t rank2[IPT / 2];  // two 16-bit ranks to a register
-    const uint32_t d0 = __shfl_sync(0xFFFFFFFFu, digit_of(key[0], shift, mask, dxor), 0);
+    uint32_t d0;
     bool differ = false;
+    if constexpr (APART) {
+      // whole keys are compared, at one operation each, and only as many as
+      // there are: by digits, all IPT of them, 2048 segments of a median of 1500
+      // u32 pairs took 140 us and take 130 (64-bit keys cost two operations a
+      // compare, so theirs go by digits after the first pass: 274 / 271)
+      const K first = __shfl_sync(0xFFFFFFFFu, key[0], 0);
+      d0 = digit_of(first, shift, mask, dxor);
+      if (KBITS == 32 || note) {
+        K bits = 0;
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) differ |= valid(i) && digit_of(key[i], shift, mask, dxor) != d0;
+        for (int i0 = 0; i0 < IPT; i0 += U) {
+          if (SPREAD && i0 >= ipt) break;
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (valid(i0 + u)) bits |= key[i0 + u] ^ first;
+        }
+        differ = ((uint32_t)(bits >> shift) & mask) != 0u;
+        if (note) {
+          bits = warp_or(bits);
+          if (lane == 0) {
+            reinterpret_cast<K*>(smem + dsum)[warp] = bits;
+            reinterpret_cast<K*>(smem + dsum)[NW + warp] = first;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int i0 = 0; i0 < IPT; i0 += U) {
+          if (SPREAD && i0 >= ipt) break;
+#pragma unroll
+          for (int u = 0; u < U; ++u) differ |= valid(i0 + u) && digit_of(key[i0 + u], shift, mask, dxor) != d0;
+        }
+      }
+    } else {
+      d0 = __shfl_sync(0xFFFFFFFFu, digit_of(key[0], shift, mask, dxor), 0);
+#pragma unroll
+      for (int i = 0; i < IPT; ++i) differ |= valid(i) && digit_of(key[i], shift, mask, dxor) != d0;
+    }
     if (__any_sync(0xFFFFFFFFu, differ)) {
       uint32_t dominant = kRadix, most = kDominantLanes - 1, position = 0;
       if constexpr (APART) {
@@ -198,7 +238,8 @@ struct SmallTile {
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
       if (valid(i)) {
-        const uint32_t p = wc[digit_of(key[i], shift, mask, dxor)] + ((i & 1) ? rank2[i / 2] >> 16 : rank2[i / 2] & 0xFFFFu);
+        const uint32_t rank = (i & 1) ? rank2[i / 2] >> 16 : rank2[i / 2] & 0xFFFFu;
+        const uint32_t p = wc[digit_of(key[i], shift, mask, dxor)] + rank;
         kb[p] = key[i];
         if (PAIRS) vb[p] = val[i];
       }
@@ -207,7 +248,22 @@ struct SmallTile {
     clear_counts(smem);
     __syncthreads();
   }
-  // A whole sort of the tile: p passes, then the store.
+  // The bits in which the tile's keys differ, as its warps noted them in a pass.
+  __device__ __forceinline__ K differing_bits(const unsigned char* smem) const {
+    const uint32_t lane = threadIdx.x & 31;
+    const K* noted = reinterpret_cast<const K*>(smem + dsum);
+    return warp_or(lane < NW && lane * keys() * 32 < count ? noted[lane] | (noted[NW + lane] ^ noted[NW]) : K(0));
+  }
+  __device__ __forceinline__ static K warp_or(K x) {
+    if constexpr (sizeof(K) == 4) return __reduce_or_sync(0xFFFFFFFFu, x);
+    return (K)__reduce_or_sync(0xFFFFFFFFu, (uint32_t)x) |
+           (K)((uint64_t)__reduce_or_sync(0xFFFFFFFFu, (uint32_t)((uint64_t)x >> 32)) << 32);
+  }
+  // A whole sort of the tile: p passes, then the store. APART: after the first
+  // pass, a place whose digit all keys share would leave them as they are and is
+  // passed over (2048 segments of a median of 1500 u32 pairs: keys below 65536
+  // 123 -> 90 us, all equal 105 -> 64, uniform words 130 / 130; the first pass
+  // is not worth a barrier of its own: 145).
   __device__ __forceinline__ void sort(unsigned char* smem, const K* keys_in, const uint32_t* vals_in, K* keys_out,
                                        uint32_t* vals_out, int places, int begin_bit, int end_bit, uint32_t top_xor,
                                        uint32_t descending, int flip) {
@@ -215,16 +271,24 @@ struct SmallTile {
     const uint32_t* vb = reinterpret_cast<const uint32_t*>(smem + vbuf);
     load_keys(keys_in, flip);
     if (kValuesFirst) load_values(vals_in);
+    K differ = ~K(0);
     for (int pass = 0; pass < places; ++pass) {
       const int shift = begin_bit + kRadixBits * pass;
       const uint32_t mask = (1u << min(kRadixBits, end_bit - shift)) - 1u;
-      if (pass > 0) load_keys(kb);
+      if (pass > 0) {
+        if (APART && ((uint32_t)(differ >> shift) & mask) == 0u) continue;
+        load_keys(kb);
+      }
       bin(
           smem, shift, mask, (pass == places - 1 ? top_xor : 0u) ^ (descending ? mask : 0u),
           [&] {
-            if (pass > 0 || !kValuesFirst) load_values(pass > 0 ? vb : vals_in);
+            if (pass > 0)
+              load_values(vb);
+            else if (!kValuesFirst)
+              load_values(vals_in);
           },
-          [](uint32_t) {});
+          [](uint32_t) {}, pass == 0);
+      if (APART && pass == 0) differ = differing_bits(smem);
     }
     for (uint32_t j = threadIdx.x; j < count; j += NT) {
       const K k = kb[j];

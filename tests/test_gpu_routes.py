@@ -189,3 +189,38 @@ def test_batches_by_blocks_an_sm(segments, kt, pairs, dist):
         ko, ek = (out[0], exp[0]) if pairs else (out, exp)
         assert np.array_equal(ko.cpu().numpy().view(ek.dtype), ek)
         assert not pairs or np.array_equal(out[1].cpu().numpy().view(np.uint32), exp[1])
+
+
+def _shared(kt, n, seed, live, odd):
+    """Uniform words of which only the bits `live` vary; with `odd`, the last key alone differs in every bit."""
+    keys = workload.keys("u64" if KB[kt] == 64 else "u32", "uniform", n, seed=seed)
+    word = workload.keys("u64" if KB[kt] == 64 else "u32", "uniform", 1, seed=seed + 1)
+    live = keys.dtype.type(live & ((1 << KB[kt]) - 1))
+    out = (keys & live) | (word[0] & ~live)
+    if odd and n:
+        out[-1] = ~out[0]
+    return out
+
+
+@pytest.mark.parametrize("live", [0, 0xFF, 0xFFFF, 0xFF00FF00, 0x00FF0000, 1 << 31, 0xFFFF << 40, 0x0F0F0F0F0F0F0F0F])
+@pytest.mark.parametrize("kt,pairs,begin,end,descending", [
+    ("u32", True, 0, 32, False), ("i32", False, 0, 32, True), ("u32", True, 3, 29, False), ("u64", True, 0, 64, False),
+    ("i64", False, 5, 61, True)])
+def test_batch_rows_that_share_places(kt, pairs, begin, end, descending, live):
+    # places that a whole segment shares are passed over, in each class, by few wide blocks or many narrow ones
+    cap = 4096 if KB[kt] == 32 else 2048
+    sizes = [1, 2, 31, 257, 300, 1000, cap - 1, cap, cap + 1, 2 * cap, 3 * cap + 5, 4 * cap]
+    for sizes in (sizes, sizes + [700] * 300, sizes + [20] * 300):
+        offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        keys = np.concatenate([_shared(kt, n, i, live, i % 3 == 2) for i, n in enumerate(sizes)])
+        vals = workload.iota_u32(keys.size)
+        key_type = osw.KEY_TYPES[kt]
+        ws = osw.batch_workspace(key_type, keys.size, len(sizes), 4 if pairs else 0, begin, end, "cuda").random_(0, 256)
+        out = osw.sort_batch(_dev(keys), torch.from_numpy(offs).cuda(), _dev(vals) if pairs else None, begin, end,
+                             key_type=kt, ws=ws, descending=descending)
+        assert osw.os_workspace_status(ws.data_ptr(), torch.cuda.current_stream().cuda_stream) == osw.OS_OK
+        exp = oracle.sort_segments(kt, keys, offs.astype(np.uint64), vals if pairs else None, begin, end,
+                                   descending=descending)
+        ko, ek = (out[0], exp[0]) if pairs else (out, exp)
+        assert np.array_equal(ko.cpu().numpy().view(ek.dtype), ek)
+        assert not pairs or np.array_equal(out[1].cpu().numpy().view(np.uint32), exp[1])
