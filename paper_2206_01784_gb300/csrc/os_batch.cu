@@ -381,23 +381,22 @@ cudaError_t launch_class(const BatchArgs& b, bool* after_kernel, cudaStream_t s)
 // first of them waits for the plan as any kernel does.
 template <int KBITS, bool PAIRS>
 cudaError_t launch_classes(const BatchArgs& b, bool* after_class, cudaStream_t s) {
-  // At most one segment an SM, and more keys than half of class 0's capacity on
-  // the mean: a segment's own time counts, so it gets a whole block of 1024
-  // threads. us a batch of u32 pairs, blocks of 256 or 512 / 1024: 16 segments
-  // of 4096 keys 30.7 / 28.7, of 8000 36.9 / 34.9 (AND of 3 words 43.0 / 34.8,
-  // 49.2 / 45.1); shorter ones leave most of the threads idle: 152 of 1000 24.6
-  // / 28.5, of 20 16.4 / 18.4; so do 64-bit keys: 152 of 4096 54.5 / 57.4, 16
-  // 47.1 / 47.1. Two segments an SM take turns: 304 of 4096 45.1 / 50.7, of 86
+  // At most one segment an SM: the longest one's own time counts, so a segment
+  // gets a whole block of 1024 threads, unless they are so short (128 keys on
+  // the mean) that most of the threads would idle. us a batch, blocks of 256 or
+  // 512 / 1024 threads: 16 segments of 4096 u32 pairs 30.7 / 28.7, 32 i32 of a
+  // median of 768 34.8 / 30.7, 30 f32 of 226 24.6 / 20.5, 16 u64 of 3584, AND of 3
+  // words, 76.7 / 69.8; short ones: 152 of 86 u32 pairs 18.5 / 19.9, u64 32.8 /
+  // 36.9. Two segments an SM take turns: 304 of 4096 u32 pairs 45.1 / 50.7, of 86
   // 28.6 / 32.8, 304 of 1000 u64 45.0 / 56.9.
-  const bool wide = KBITS == 32 && b.num_segments <= (uint32_t)device_sm_count() &&
-                    b.n_total >= (uint64_t)b.num_segments * (b.class_max[0] / 2);
+  const bool wide = b.num_segments <= (uint32_t)device_sm_count() && b.n_total >= 128ull * b.num_segments;
   cudaError_t e = launch_class<KBITS, PAIRS, 2, false>(b, after_class, s);
-  if constexpr (KBITS == 32) {
-    if (e == cudaSuccess && wide) e = launch_class<KBITS, PAIRS, 1, true>(b, after_class, s);
-    if (e == cudaSuccess && wide) e = launch_class<KBITS, PAIRS, 0, true>(b, after_class, s);
-  }
-  if (e == cudaSuccess && !wide) e = launch_class<KBITS, PAIRS, 1, false>(b, after_class, s);
-  if (e == cudaSuccess && !wide) e = launch_class<KBITS, PAIRS, 0, false>(b, after_class, s);
+  if (e == cudaSuccess)
+    e = wide ? launch_class<KBITS, PAIRS, 1, true>(b, after_class, s)
+             : launch_class<KBITS, PAIRS, 1, false>(b, after_class, s);
+  if (e == cudaSuccess)
+    e = wide ? launch_class<KBITS, PAIRS, 0, true>(b, after_class, s)
+             : launch_class<KBITS, PAIRS, 0, false>(b, after_class, s);
   return e;
 }
 
