@@ -412,7 +412,7 @@ int run_histogram(const Plan& plan, int key_type, const void* keys, uint64_t n, 
 bool run_small(const Plan& plan, int key_type, const void* keys_in, void* keys_out, const uint32_t* vals_in,
                uint32_t* vals_out, uint64_t n, int begin_bit, int end_bit, char* w, cudaStream_t s, int* rc) {
   if (plan.radix_bits != kRadixBits || plan.strips != 1 || plan.fault_tile >= 0) return false;
-  const int form = small_form(plan.key_bits, plan.pairs, n, device_sm_count());
+  const int form = small_form(plan.key_bits, n, device_sm_count());
   if (form == 0) return false;
   const uint32_t blocks = small_blocks(form, n);
   const os_workspace_layout& L = plan.layout;
@@ -611,8 +611,8 @@ struct BatchPlan {
   uint64_t max_large = 0;    // segments beyond the one-block sorts
   uint64_t max_tiles = 0, max_items = 0;  // capacities (any tile geometry)
   uint64_t grid_tiles = 0;   // tiles at most, with this plan's tile
-  size_t seg_done = 0, seg_hist = 0, zero_end = 0, seg_rank_words = 0, seg_bin_offsets = 0, large_range = 0, tile_base = 0;
-  size_t hist_base = 0, class_list = 0, hist_large = 0, tile_desc = 0, status[2] = {0, 0};
+  size_t seg_done = 0, seg_hist = 0, zero_end = 0, seg_rank_words = 0, seg_bin_offsets = 0, large_range = 0;
+  size_t tile_base = 0, hist_base = 0, class_list = 0, hist_large = 0, tile_desc = 0, status[2] = {0, 0};
   size_t alt_keys = 0, alt_vals = 0, total = 0;
 };
 
@@ -651,7 +651,8 @@ int make_batch_plan(int key_type, uint64_t n_total, int64_t num_segments, int va
   bp->tile = tile_keys_for(kb, bp->pairs, bp->cfg);
   const uint32_t min_tile = min_tile_keys(kb, bp->pairs);
   // (n_total keys that fit the last class make no large segment)
-  bp->max_large = n_total > batch_class_capacity(kb, kBatchClasses - 1) ? n_total / (batch_class_capacity(kb, 0) + 1) : 0;
+  const uint32_t one_block = batch_class_capacity(kb, kBatchClasses - 1);
+  bp->max_large = n_total > one_block ? n_total / (batch_class_capacity(kb, 0) + 1) : 0;
   if (bp->max_large > S) bp->max_large = S;
   bp->max_tiles = n_total / min_tile + bp->max_large;
   bp->grid_tiles = n_total / bp->tile + bp->max_large;

@@ -152,7 +152,7 @@ struct TileCtx {
   uint32_t out_base;     // array index of the chain's (segment's) first key
   uint32_t out_len;      // keys in the chain's segment
   uint32_t bulk;         // staged by bulk copies (wait on the mbarriers)
-  uint32_t rank_word;    // how this place (of this segment) is ranked (rank_word in os_common.cuh)
+  uint32_t rank_word;    // how this place (of this segment) is ranked (finish_place in os_common.cuh)
   const uint32_t* bin_offsets;  // this place's 256 bin offsets (segment-relative)
 };
 

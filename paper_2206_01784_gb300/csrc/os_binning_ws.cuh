@@ -49,9 +49,9 @@ namespace onesweep {
 // tiles; kept as a variant that a caller or the autotuner may name.
 //
 // Shapes of the persistent kernel: ranker warps, keys per ranker thread and
-// writer warps (measured with ballots and lane masks on GB300 at 2^28 u32 pairs: 24 rankers x 8 keys with
-// 8 writers 1.415 ms per pass, 16 x 12 with 8 writers 1.434, with 16 writers
-// 1.462). Shared memory holds one staging buffer and two sorted buffers of a
+// writer warps (measured with ballots and lane masks on GB300 at 2^28 u32
+// pairs: 24 rankers x 8 keys with 8 writers 1.415 ms per pass, 16 x 12 with 8
+// writers 1.434, with 16 writers 1.462). Shared memory holds one staging buffer and two sorted buffers of a
 // tile, plus the rankers' per-warp digit tables.
 template <int KBITS, bool PAIRS> struct WsShape;
 template <> struct WsShape<32, true> { static constexpr int NR = 24, IPT = 8, NWR = 8; };    // 6144-key tiles

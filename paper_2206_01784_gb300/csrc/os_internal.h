@@ -44,7 +44,7 @@ struct HistArgs {
   uint32_t* done_counter;    // zeroed by the caller (device)
   uint32_t* clear;           // words to zero on the way (status slab of pass 0), may be null
   uint64_t clear_words;
-  uint32_t* rank_words;      // [p] how each place's digits are ranked (rank_word; may be null)
+  uint32_t* rank_words;      // [p] how each place's digits are ranked (finish_place; may be null)
   uint32_t top_xor;          // signed keys: high bit of the top place's digit inverted (else 0)
   uint32_t descending;       // offsets (and the reported histograms) for complemented digits
 };
@@ -120,7 +120,7 @@ struct SmallArgs {
 
 // Form of the one-launch sort for n keys on a device of `sms` SMs; 0: none
 // (the array is too large for it). small_blocks: its blocks.
-int small_form(int key_bits, bool pairs, uint64_t n, int sms);
+int small_form(int key_bits, uint64_t n, int sms);
 uint32_t small_blocks(int form, uint64_t n);
 bool small_needs_matrices(int form);  // exchanges counts through SmallArgs::counts_*
 cudaError_t launch_small(int key_bits, bool pairs, int form, const SmallArgs& a, cudaStream_t s);

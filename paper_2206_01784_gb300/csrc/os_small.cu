@@ -53,8 +53,9 @@ struct SmallLayout {
   static constexpr size_t scan = Tile::smem_bytes;                        // [8] scan scratch
   static constexpr size_t gtot = scan + 32;                               // [256] digit totals of all blocks
   static constexpr size_t glow = gtot + kRadix * 4;                       // [256] ... of the lower blocks, then bin bases
-  static constexpr size_t rows = glow + kRadix * 4;                       // cluster: [16][256] counts of each block
-  static constexpr size_t krecv = rows + (kCluster ? (size_t)kMaxCluster * kRadix * 4 : 0);  // cluster: the next pass's tile
+  // cluster: [16][256] counts of each block, then the next pass's tile
+  static constexpr size_t rows = glow + kRadix * 4;
+  static constexpr size_t krecv = rows + (kCluster ? (size_t)kMaxCluster * kRadix * 4 : 0);
   static constexpr size_t vrecv = krecv + (kCluster ? (size_t)Tile::T * sizeof(typename Tile::K) : 0);
   static constexpr size_t smem_bytes =
       SCOPE == kScopeBlock ? Tile::smem_bytes : vrecv + (kCluster && PAIRS ? (size_t)Tile::T * 4 : 0);
@@ -339,6 +340,13 @@ cudaError_t launch_small_t(const SmallArgs& a, cudaStream_t s) {
 // cycles per warp) are slower than a grid's way through L2 (65536 keys: 32.8
 // against 24.6). 64-bit pairs: 1000 keys 10.3, 16384 34.9, 300000 51.3, 2^20
 // 96.
+// Those are uniform words. Keys whose digits repeat meet in the counters here,
+// where the passes go over to votes, and gain less or lose at the top of the
+// range (one launch / the passes; the AND of 3 words, of 5, all equal): 150 000
+// u32 pairs 31 / 39, 29 / 39, 23 / 30; 2^20 57 / 70, 55 / 61, 35 / 41; 1.87M 76 /
+// 76, 74 / 65, 43 / 45 (uniform 57 / 66); u64 pairs, 2^20 123 / 106, 121 / 99, 74 /
+// 78 (uniform 96 / 104). Setting a frequent digit apart, as a batch's sorts do,
+// costs uniform words about 1 us a pass; a lower limit costs them 7 to 15 %.
 struct SmallForm {
   uint32_t tile;
   int scope;
@@ -374,8 +382,7 @@ cudaError_t launch_small_kp(int form, const SmallArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-int small_form(int key_bits, bool pairs, uint64_t n, int sms) {
-  (void)pairs;
+int small_form(int key_bits, uint64_t n, int sms) {
   if (n == 0 || sms <= 0) return 0;
   if (sms > kMaxGrid) sms = kMaxGrid;
   for (int f = 1; f <= kSmallForms; ++f) {
