@@ -95,7 +95,7 @@ def workload_name(n, dist, seed, pairs=True, key_type="u32"):
 
 # The sources the timed binning kernel is compiled from: a profile's traffic
 # figure stays valid while these are unchanged.
-KERNEL_SOURCES = ("os_common.cuh", "os_internal.h", "os_binning.cuh", "os_bin32_pairs_f0_single.cu")
+KERNEL_SOURCES = ("os_common.cuh", "os_internal.h", "os_places.h", "os_binning.cuh", "os_bin32_pairs_f0_single.cu")
 
 
 def source_hash() -> str:
